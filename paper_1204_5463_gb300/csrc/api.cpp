@@ -56,7 +56,7 @@ cudaEvent_t Profiler::take() {
     return e;
 }
 
-int Profiler::begin(const char* name, double bytes, cudaEvent_t* start_out, int* idx) {
+int Profiler::begin(const char* name, double bytes, cudaEvent_t* start_out, int* idx, int count) {
     int i = 0;
     for (; i < (int)k.size(); ++i)
         if (k[i].name == name) break;
@@ -70,6 +70,7 @@ int Profiler::begin(const char* name, double bytes, cudaEvent_t* start_out, int*
     *start_out = a;
     *idx = i;
     k[i].pending_bytes.push_back(bytes);
+    k[i].pending_count.push_back(count);
     return 0;
 }
 
@@ -90,13 +91,14 @@ void Profiler::drain() {
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e.pending[i].first, e.pending[i].second);
             e.total_ms += ms;
-            e.launches += 1;
+            e.launches += (i < e.pending_count.size()) ? e.pending_count[i] : 1;
             e.bytes += (i < e.pending_bytes.size()) ? e.pending_bytes[i] : 0.0;
             pool.push_back(e.pending[i].first);
             pool.push_back(e.pending[i].second);
         }
         e.pending.clear();
         e.pending_bytes.clear();
+        e.pending_count.clear();
     }
 }
 
@@ -158,10 +160,77 @@ int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char
     return DW_OK;
 }
 
+size_t sap_state_bytes(int prec, const Geom& g) {
+    const bool half = (prec == P16 || prec == PB16);
+    return (size_t)spinor_bytes(prec == P64 ? P64 : P32, g.V) * (half ? 2 : 1);
+}
+
+size_t sap_inbox_bytes(int prec, const Geom& g) {
+    return (size_t)g.ndom * sap_inbox_slots(g) * 12 * (prec == P64 ? 8 : 4);
+}
+
+// the table of inbox slots and, behind it, the barrier counters
+static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** bar) {
+    const size_t fbytes = ((size_t)sap_inbox_slots(ctx->g) / 2 * sizeof(unsigned short) + 15) / 16 * 16;
+    const size_t cbytes = 2 * DW_MAX_RHS * sizeof(unsigned);
+    int rc;
+    if (!ctx->sap_faces.p) {
+        std::vector<unsigned short> f;
+        sap_faces(ctx->g, &f);
+        if ((rc = ctx->sap_faces.ensure(fbytes + cbytes))) return rc;
+        DW_CUDA_TRY(cudaMemcpyAsync(ctx->sap_faces.p, f.data(), f.size() * sizeof(f[0]), cudaMemcpyHostToDevice,
+                                    ctx->stream));
+        DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    }
+    *faces = ctx->sap_faces.as<unsigned short>();
+    *bar = reinterpret_cast<unsigned*>(ctx->sap_faces.as<char>() + fbytes);
+    if (!ctx->sap_counters_ok) {
+        DW_CUDA_TRY(cudaMemsetAsync(*bar, 0, cbytes, ctx->stream));
+        ctx->sap_counters_ok = true;
+    }
+    return DW_OK;
+}
+
+int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
+            long long inbox_rs, const int* jtab, int nrhs, int nact, int ncycles, int nmr) {
+    const Geom& g = ctx->g;
+    const long long sb = spinor_bytes(prec, g.V);
+    const double first = 0.5 * ((double)nact * 2.0 * sb + link_bytes(prec, g.V));
+    const double next = 0.5 * ((double)nact * 3.0 * sb + link_bytes(prec, g.V));
+    const char *U, *Uimg;
+    int rc;
+    if (sap_apply_fits(prec, g)) {
+        if ((rc = sap_links_for(ctx, prec, 0, &U, &Uimg))) return rc;
+        SapWork w;
+        w.Uimg = Uimg;
+        w.rho = state;
+        w.rho_rs = w.xpart_rs = state_rs;
+        w.xpart = state + spinor_bytes(P32, g.V);
+        w.inbox = inbox;
+        w.inbox_rs = inbox_rs;
+        w.err = ctx->sap_err.d;
+        if ((rc = sap_tables_for(ctx, &w.faces, &w.bar))) return rc;
+        return launch_sap_apply(prec, g, ctx->m0, v, x, w, jtab, nrhs, ncycles, nmr, ctx->stream, ctx->clover(),
+                                &ctx->prof, first, next);
+    }
+    const int thr = ctx->sap_threads[prec];
+    if ((rc = sap_links_for(ctx, prec, thr, &U, &Uimg))) return rc;
+    for (int cyc = 0; cyc < ncycles; ++cyc)
+        for (int colour = 0; colour < 2; ++colour) {
+            const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
+            ProfScope ps(&ctx->prof, "sap_sweep", mode == 2 ? next : first);
+            if ((rc = launch_sap_sweep(prec, prec, g, ctx->m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, thr,
+                                       ctx->stream, ctx->clover(), ctx->sap_err.d)))
+                return rc;
+        }
+    return DW_OK;
+}
+
 int sap_check(dw_ctx* ctx) {
     if (!ctx->sap_err.h || *reinterpret_cast<volatile int*>(ctx->sap_err.h) == 0) return DW_OK;
     *reinterpret_cast<volatile int*>(ctx->sap_err.h) = 0;
-    return fail(DW_ETIMEOUT, "a SAP domain's bulk copy of its links did not complete");
+    ctx->sap_counters_ok = false;
+    return fail(DW_ETIMEOUT, "a bounded wait of the SAP preconditioner gave up");
 }
 
 static int check_prec(int p) { return (p >= 0 && p <= 3) ? DW_OK : fail(DW_EINVAL, "bad precision"); }
@@ -211,7 +280,7 @@ int dw_create(const dw_lattice* L, void* cuda_stream, dw_ctx** out) {
         return fail(DW_ECUDA, std::string("no CUDA device: ") + cudaGetErrorString(e));
     }
     c->sap_threads.assign(4, 0);
-    for (auto* b : {&c->U[0], &c->U[1], &c->U[2], &c->U[3], &c->U[4], &c->work_in, &c->work_out, &c->work_aux,
+    for (auto* b : {&c->U[0], &c->U[1], &c->U[2], &c->U[3], &c->U[4], &c->work_in, &c->work_out, &c->work_aux, &c->work_sap, &c->sap_faces,
                    &c->Uimg[0], &c->Uimg[1], &c->Uimg[2], &c->Uimg[3]})
         b->st = c->stream;
     *out = c;
@@ -313,21 +382,16 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     const long long V = ctx->g.V;
     const long long fb = spinor_bytes(storage, V);
     int rc;
-    const char *U, *Uimg;
-    if ((rc = sap_links_for(ctx, storage, ctx->sap_threads[storage], &U, &Uimg))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = ctx->work_out.ensure((size_t)nrhs * fb))) return rc;
+    const size_t sbytes = sap_state_bytes(storage, ctx->g), ibytes = sap_inbox_bytes(storage, ctx->g);
+    if (sap_apply_fits(storage, ctx->g) && (rc = ctx->work_sap.ensure((size_t)nrhs * (sbytes + ibytes)))) return rc;
+    char* scratch = ctx->work_sap.as<char>();
     if ((rc = launch_to_internal(storage, v, ctx->work_in.as<char>(), V, nrhs, ctx->stream))) return rc;
     FieldRef fv{ctx->work_in.as<char>(), fb, 0, 0}, fx{ctx->work_out.as<char>(), fb, 0, 0};
-    for (int cyc = 0; cyc < ncycles; ++cyc)
-        for (int colour = 0; colour < 2; ++colour) {
-            const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
-            ProfScope ps(&ctx->prof, "sap_sweep",
-                         (double)nrhs * 0.5 * (2.0 * fb + (mode == 2 ? fb : 0) + link_bytes(storage, V)));
-            if ((rc = launch_sap_sweep(storage, storage, ctx->g, ctx->m0, fv, fx, Uimg, nullptr, nrhs, colour, nmr,
-                                       mode, ctx->sap_threads[storage], ctx->stream, ctx->clover(), ctx->sap_err.d)))
-                return rc;
-        }
+    if ((rc = sap_run(ctx, storage, fv, fx, scratch, (long long)sbytes, scratch + nrhs * sbytes, (long long)ibytes,
+                      nullptr, nrhs, nrhs, ncycles, nmr)))
+        return rc;
     if ((rc = launch_from_internal(storage, ctx->work_out.as<char>(), z, V, nrhs, ctx->stream))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return sap_check(ctx);

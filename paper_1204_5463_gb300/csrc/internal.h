@@ -71,11 +71,12 @@ struct DevBuf {
 // while profiling is switched on.
 struct KernelProfile {
     std::string name;
-    long long launches = 0;
+    long long launches = 0;  // units of work: launches, or the SAP sweeps that one launch runs
     double total_ms = 0.0;
     double bytes = 0.0;  // algorithmic bytes summed over launches
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending;
     std::vector<double> pending_bytes;
+    std::vector<int> pending_count;
 };
 
 struct Profiler {
@@ -84,7 +85,7 @@ struct Profiler {
     std::vector<cudaEvent_t> pool;  // recycled events (creation is not free)
     cudaStream_t stream = nullptr;
     cudaEvent_t take();
-    int begin(const char* name, double bytes, cudaEvent_t* start_out, int* idx);
+    int begin(const char* name, double bytes, cudaEvent_t* start_out, int* idx, int count = 1);
     void end(int idx, cudaEvent_t start);
     void drain();  // turn pending event pairs into totals (synchronises)
     void reset();
@@ -96,8 +97,8 @@ struct ProfScope {
     Profiler* p;
     int idx = -1;
     cudaEvent_t start = nullptr;
-    ProfScope(Profiler* prof, const char* name, double bytes) : p(prof) {
-        if (p && p->on) p->begin(name, bytes, &start, &idx);
+    ProfScope(Profiler* prof, const char* name, double bytes, int count = 1) : p(prof) {
+        if (p && p->on) p->begin(name, bytes, &start, &idx, count);
     }
     ~ProfScope() {
         if (p && p->on && idx >= 0) p->end(idx, start);
@@ -144,7 +145,10 @@ struct dw_ctx {
     dwk::ClovRef clov{nullptr, nullptr};
     dwk::DevBuf Uimg[4];            // SAP links per domain as shared-memory images (per storage precision)
     int Uimg_threads[4] = {0, 0, 0, 0};  // CTA size the image was packed for (0: none)
-    dwk::HostFlag sap_err;          // set by a SAP sweep whose link copy did not complete
+    dwk::HostFlag sap_err;          // set by a SAP kernel whose bounded wait gave up
+    dwk::DevBuf sap_faces;          // inbox slots of a domain (sap_faces()), with the barrier counters behind them
+    bool sap_counters_ok = false;   // the barrier counters are zero (cleared after a wait that gave up)
+    dwk::DevBuf work_sap;           // scratch of sap_precondition
     std::atomic<int> cancel{0};     // set by dw_cancel; the running solve stops before its next step
     const dwk::ClovRef* clover() const { return csw != 0.0 ? &clov : nullptr; }
 };
@@ -189,7 +193,37 @@ int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, in
 // links of precision prec in both layouts for a sweep of `threads` threads
 // (the image is packed on first use and after dw_set_gauge), and the error flag
 int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char** img);
-// after the stream was synchronised: DW_ETIMEOUT if a SAP link copy gave up
+// ----- sap_apply.cu --------------------------------------------------------
+// z = M v with the domains' residuals carried along (sap_apply.cu), for
+// domains that sap_apply_fits accepts. Per right-hand side: rho (the residuals,
+// spinor layout of the arithmetic precision), xpart (the same size, only for
+// 16-bit storage) and the inboxes.
+struct SapWork {
+    const char* Uimg;
+    const unsigned short* faces;
+    char *rho, *xpart, *inbox;
+    long long rho_rs, xpart_rs, inbox_rs;
+    unsigned* bar;
+    int* err;
+};
+bool sap_apply_fits(int prec, const Geom& g);
+int sap_apply_smem(int pspin, int plink, const Geom& g);
+int sap_inbox_slots(const Geom& g);
+void sap_faces(const Geom& g, std::vector<unsigned short>* out);
+int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab,
+                     int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
+                     double bytes_first, double bytes_next);
+// Scratch of one application and right-hand side in two pieces: the residuals
+// (with the 16-bit formats' iterate behind them) and the inboxes. Neither
+// exceeds a double-precision field (192 bytes per site).
+size_t sap_state_bytes(int prec, const Geom& g);
+size_t sap_inbox_bytes(int prec, const Geom& g);
+// the whole application, nact of the nrhs right-hand sides active: by
+// launch_sap_apply where the domain fits, else sweep by sweep (the scratch is
+// then unused); state and inbox: scratch of the strides given
+int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
+            long long inbox_rs, const int* jtab, int nrhs, int nact, int ncycles, int nmr);
+// after the stream was synchronised: DW_ETIMEOUT if a SAP kernel's bounded wait gave up
 int sap_check(dw_ctx* ctx);
 
 // ----- blas.cu -------------------------------------------------------------

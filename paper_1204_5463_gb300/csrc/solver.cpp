@@ -69,9 +69,9 @@ struct Solver {
     long long fv;       // bytes of one basis vector in format vp
     int NP;             // multi-dot row length (m + 2)
     int nblk;
-    const char *U_sap, *U_sap_img, *U_mv, *U64;
+    const char *U_mv, *U64;
     // device buffers (owned by the workspace of the context)
-    char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap;
+    char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap, *canon;
     double2 *partial, *dots, *Qd, *etad;
     unsigned* cnt_d;  // reduction counters of the multi-dot and multi-axpy launches
     double *norm2d, *scal_d;
@@ -206,9 +206,8 @@ int Solver::setup() {
     NP = m + 2;
     nblk = blas_nblk(n);
     int rc;
-    if ((rc = sap_links_for(ctx, sp, (ctx->sap_threads.size() > (size_t)sp) ? ctx->sap_threads[sp] : 0, &U_sap,
-                            &U_sap_img)))
-        return rc;
+    const char *U_sap, *U_sap_img;  // the preconditioner's links, before the first step needs them
+    if ((rc = sap_links_for(ctx, sp, ctx->sap_threads[sp], &U_sap, &U_sap_img))) return rc;
     if ((rc = gauge_for(ctx, mp == P64 ? P64 : P32, &U_mv))) return rc;
     // explicit residual: FP64 links for FP64 outer vectors, double-float links otherwise
     if ((rc = gauge_for(ctx, op == PDF ? PDF : P64, &U64))) return rc;
@@ -222,6 +221,9 @@ int Solver::setup() {
     if ((rc = W->r.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = W->vlow.ensure((size_t)nrhs * sb))) return rc;
     if (vp != op && (rc = W->rlow.ensure((size_t)nrhs * fv))) return rc;
+    // the caller's layout of the right-hand sides; between the set-up and the
+    // end of a solve it holds the preconditioner's inboxes
+    if ((rc = W->canon.ensure((size_t)nrhs * 24 * V * sizeof(double)))) return rc;
     if ((rc = W->zscr.ensure((size_t)(k > 0 ? k : 1) * zb))) return rc;
     if ((rc = W->partial.ensure((size_t)nrhs * nblk * NP * sizeof(double2)))) return rc;
     // per-rhs counters of the multi-dot and multi-axpy launches (their last CTA
@@ -260,6 +262,7 @@ int Solver::setup() {
     rb = W->r.as<char>();
     vlow = W->vlow.as<char>();
     zscr = W->zscr.as<char>();
+    canon = W->canon.as<char>();
     zsap = (zp != sp) ? W->zsap.as<char>() : nullptr;
     rlow = (vp != op) ? W->rlow.as<char>() : nullptr;
     partial = W->partial.as<double2>();
@@ -500,16 +503,11 @@ int Solver::step() {
     const FieldRef Lf{vlow, sb, 0, 0};
     const FieldRef Zs = (zp == sp) ? Zf : FieldRef{zsap, sb, 0, 0};  // where the SAP writes z_j
     // z_j = M v_j  (v_j was written in SAP storage to vlow when it was normalised)
-    for (int cyc = 0; cyc < P.sap_cycles; ++cyc)
-        for (int colour = 0; colour < 2; ++colour) {
-            const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
-            const double bytes = (double)nact * 0.5 * (2.0 * sb + (mode == 2 ? sb : 0) + link_bytes(sp, V));
-            ProfScope ps(&ctx->prof, "sap_sweep", bytes);
-            const int thr = (ctx->sap_threads.size() > (size_t)sp) ? ctx->sap_threads[sp] : 0;
-            if ((rc = launch_sap_sweep(sp, sp, g, ctx->m0, Lf, Zs, U_sap_img, jtab_d, nrhs, colour, P.mr_steps,
-                                       mode, thr, st, ctx->clover(), ctx->sap_err.d)))
-                return rc;
-        }
+    // The preconditioner's scratch lies in rb (the explicit residual is formed
+    // and consumed within cycle_end, so rb is free during the steps) and in the
+    // staging copy of the right-hand sides: 192 bytes per site and rhs each.
+    if ((rc = sap_run(ctx, sp, Lf, Zs, rb, fb, canon, 192 * V, jtab_d, nrhs, nact, P.sap_cycles, P.mr_steps)))
+        return rc;
     if (zp != sp) {
         ProfScope ps(&ctx->prof, "z_widen", (double)nact * (sb + zb));
         if ((rc = launch_convert(sp, zp, Zs, Zf, V, jtab_d, nrhs, st))) return rc;
@@ -656,7 +654,6 @@ int Solver::run(const double* b_user, double* x_user, dw_stats* S, const std::at
     const double* b_dev = b_user;
     double* x_dev = x_user;
     if (P.host_buffers) {
-        if ((rc = W->canon.ensure(canon_bytes))) return rc;
         DW_CUDA_TRY(cudaMemcpyAsync(W->canon.p, b_user, canon_bytes, cudaMemcpyHostToDevice, st));
         b_dev = W->canon.as<double>();
     }
