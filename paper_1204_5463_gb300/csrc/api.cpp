@@ -152,21 +152,14 @@ int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char
     threads = sap_threads(ctx->g, threads);
     if (ctx->Uimg_threads[prec] != threads) {
         if ((rc = ctx->Uimg[prec].ensure(sap_link_image_bytes(prec, ctx->g, threads)))) return rc;
-        if ((rc = launch_sap_link_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), threads, ctx->stream)))
-            return rc;
+        rc = sap_apply_fits(prec, ctx->g)
+                 ? launch_sap_apply_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), ctx->stream)
+                 : launch_sap_link_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), threads, ctx->stream);
+        if (rc) return rc;
         ctx->Uimg_threads[prec] = threads;
     }
     *img = ctx->Uimg[prec].as<char>();
     return DW_OK;
-}
-
-size_t sap_state_bytes(int prec, const Geom& g) {
-    const bool half = (prec == P16 || prec == PB16);
-    return (size_t)spinor_bytes(prec == P64 ? P64 : P32, g.V) * (half ? 2 : 1);
-}
-
-size_t sap_inbox_bytes(int prec, const Geom& g) {
-    return (size_t)g.ndom * sap_inbox_slots(g) * 12 * (prec == P64 ? 8 : 4);
 }
 
 // the table of inbox slots and, behind it, the barrier counters
@@ -175,12 +168,8 @@ static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** 
     const size_t cbytes = 2 * DW_MAX_RHS * sizeof(unsigned);
     int rc;
     if (!ctx->sap_faces.p) {
-        std::vector<unsigned short> f;
-        sap_faces(ctx->g, &f);
         if ((rc = ctx->sap_faces.ensure(fbytes + cbytes))) return rc;
-        DW_CUDA_TRY(cudaMemcpyAsync(ctx->sap_faces.p, f.data(), f.size() * sizeof(f[0]), cudaMemcpyHostToDevice,
-                                    ctx->stream));
-        DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        if ((rc = launch_sap_faces(ctx->g, ctx->sap_faces.as<unsigned short>(), ctx->stream))) return rc;
     }
     *faces = ctx->sap_faces.as<unsigned short>();
     *bar = reinterpret_cast<unsigned*>(ctx->sap_faces.as<char>() + fbytes);

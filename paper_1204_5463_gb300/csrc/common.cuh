@@ -427,10 +427,10 @@ __device__ __forceinline__ void load_link(const char* base, long long V, int mu,
 // U^dagger, conj(w) h = w.re h + w.im (-i h)). It saves issue slots where the
 // registers allow (the SAP sweeps: 5% faster batched); in the stand-alone
 // stencil, capped at 64-80 registers, it spills and loses.
-template <class C, bool DAG, bool PACK = false>
+template <class C, bool DAG, int PACK = 0>
 __device__ __forceinline__ void su3_mul(const cx<C> u[9], const cx<C> h[3], cx<C> k[3]) {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
-    if constexpr (PACK && std::is_same<C, float>::value) {
+    if constexpr (PACK == 1 && std::is_same<C, float>::value) {
         float2 hp[3], hr[3];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
@@ -451,6 +451,25 @@ __device__ __forceinline__ void su3_mul(const cx<C> u[9], const cx<C> h[3], cx<C
         return;
     }
 #endif
+    if constexpr (PACK == 2) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const cx<C> w0 = DAG ? u[a] : u[3 * a];
+            C re = w0.re * h[0].re, im = w0.re * h[0].im;
+            re = fma(DAG ? w0.im : -w0.im, h[0].im, re);
+            im = fma(DAG ? -w0.im : w0.im, h[0].re, im);
+#pragma unroll
+            for (int b = 1; b < 3; ++b) {
+                const cx<C> w = DAG ? u[3 * b + a] : u[3 * a + b];
+                re = fma(w.re, h[b].re, re);
+                im = fma(w.re, h[b].im, im);
+                re = fma(DAG ? w.im : -w.im, h[b].im, re);
+                im = fma(DAG ? -w.im : w.im, h[b].re, im);
+            }
+            k[a] = mk<C>(re, im);
+        }
+        return;
+    }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         cx<C> acc;
@@ -480,10 +499,10 @@ __device__ __forceinline__ cx<float> fma_pair(float2 w, float2 b, cx<float> a) {
 #endif
 
 // upper two spin rows of (1 + SIGN gamma_MU) psi
-template <int MU, int SIGN, class C, bool PACK = false>
+template <int MU, int SIGN, class C, int PACK = 0>
 __device__ __forceinline__ void project(const cx<C> psi[12], cx<C> h0[3], cx<C> h1[3]) {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
-    if constexpr (PACK && std::is_same<C, float>::value) {
+    if constexpr (PACK == 1 && std::is_same<C, float>::value) {
         const float s = (float)SIGN;
         const float2 pp = make_float2(s, s), pm = make_float2(s, -s), mp = make_float2(-s, s),
                      mm = make_float2(-s, -s);
@@ -528,10 +547,10 @@ __device__ __forceinline__ void project(const cx<C> psi[12], cx<C> h0[3], cx<C> 
 }
 
 // acc += the four spin rows rebuilt from the multiplied upper rows k0, k1
-template <int MU, int SIGN, class C, bool PACK = false>
+template <int MU, int SIGN, class C, int PACK = 0>
 __device__ __forceinline__ void reconstruct(const cx<C> k0[3], const cx<C> k1[3], cx<C> acc[12]) {
 #if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
-    if constexpr (PACK && std::is_same<C, float>::value) {
+    if constexpr (PACK == 1 && std::is_same<C, float>::value) {
         const float s = (float)SIGN;
         const float2 pp = make_float2(s, s), pm = make_float2(s, -s), mp = make_float2(-s, s),
                      mm = make_float2(-s, -s);
@@ -577,7 +596,7 @@ __device__ __forceinline__ void reconstruct(const cx<C> k0[3], const cx<C> k1[3]
     }
 }
 
-template <int MU, int SIGN, class C, bool PACK = false>
+template <int MU, int SIGN, class C, int PACK = 0>
 __device__ __forceinline__ void hop(const cx<C> psi[12], const cx<C> u[9], cx<C> acc[12]) {
     cx<C> h0[3], h1[3], k0[3], k1[3];
     project<MU, SIGN, C, PACK>(psi, h0, h1);

@@ -146,7 +146,7 @@ struct dw_ctx {
     dwk::DevBuf Uimg[4];            // SAP links per domain as shared-memory images (per storage precision)
     int Uimg_threads[4] = {0, 0, 0, 0};  // CTA size the image was packed for (0: none)
     dwk::HostFlag sap_err;          // set by a SAP kernel whose bounded wait gave up
-    dwk::DevBuf sap_faces;          // inbox slots of a domain (sap_faces()), with the barrier counters behind them
+    dwk::DevBuf sap_faces;          // inbox slots of a domain (launch_sap_faces), with the barrier counters behind them
     bool sap_counters_ok = false;   // the barrier counters are zero (cleared after a wait that gave up)
     dwk::DevBuf work_sap;           // scratch of sap_precondition
     std::atomic<int> cancel{0};     // set by dw_cancel; the running solve stops before its next step
@@ -209,7 +209,8 @@ struct SapWork {
 bool sap_apply_fits(int prec, const Geom& g);
 int sap_apply_smem(int pspin, int plink, const Geom& g);
 int sap_inbox_slots(const Geom& g);
-void sap_faces(const Geom& g, std::vector<unsigned short>* out);
+int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st);
+int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st);
 int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab,
                      int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
                      double bytes_first, double bytes_next);

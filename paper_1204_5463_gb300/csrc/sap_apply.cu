@@ -25,11 +25,13 @@
 // (5.3 us of a 22 us sweep), and a launch per sweep costs 8-9 us between the
 // sweeps of 256 domains. Here the residual takes 1.8 us, and the sends 1.2 us.
 // Measured against one launch of sap_sweep_kernel per sweep (5 cycles x 4 MR
-// steps unless stated): 8^3 x 16, 2 rhs served on 4 streams 37.4 -> 30.9 ms a
-// burst; 12^3 x 18 in 3^4 domains, 3 BF16 rhs 343 -> 298 us; 24^3 x 48, 12 FP16
-// rhs 14.92 -> 13.50 ms; 16^3 x 32 FP32 343 -> 332 us, with the clover term (8
-// x 5) 767 -> 687 us. Four fifths of the rest are the MR steps: 5600 cycles a
-// step for the one domain of an SM, 9600 for two.
+// steps unless stated): 8^3 x 16, 2 rhs served on 4 streams 38.2 -> 29.4 ms a
+// burst; 12^3 x 18 in 3^4 domains, 3 BF16 rhs (4 x 5) 341 -> 289 us; 24^3 x 48,
+// 12 FP16 rhs 14.91 -> 12.87 ms; 16^3 x 32 FP32 342 -> 314 us, with the clover
+// term (8 x 5) 766 -> 641 us. Four fifths of that are the MR steps: 4800 cycles
+// a step for the one domain of an SM, 7700 for two, of which the shared-memory
+// pipe is busy 5900 (367 wavefronts a warp and step); paired, scalar and mixed
+// forms of the hop's FP32 arithmetic are all within 2% of one another.
 #include <map>
 #include <mutex>
 
@@ -40,19 +42,21 @@ namespace dwk {
 
 namespace {
 
+constexpr int kChain = 2;  // su3_mul as chains of scalar FMAs
+
 template <class C>
 struct SapArgs {
     Geom g;
     C diag;
     FieldRef v, x;
-    const char* Uimg;             // links of every domain as the shared-memory image of LinkSh
-    const unsigned short* faces;  // [ns]: lower-face site | mu << 10 of an inbox slot
+    const char* Uimg;             // links of every domain as the shared-memory image of LinkWarp
+    const unsigned short* faces;  // [ns / 2]: lower-face site | mu << 10 of an inbox slot
     int ns;                       // inbox slots per domain (two per face site and direction)
     char* rho;                    // per rhs: the domains' residuals, site layout of the arithmetic type
     long long rho_rs;
     char* xpart;                  // per rhs: the iterate between cycles, same layout
     long long xpart_rs;
-    char* inbox;                  // per rhs: [domain][plane][slot]
+    char* inbox;                  // per rhs: [domain] of Half<C> boxes
     long long inbox_rs;
     const int* jtab;
     int nrhs, nmr;
@@ -83,54 +87,180 @@ __device__ __forceinline__ void state_load(const char* base, long long V, long l
     }
 }
 
-// a half spinor (upper two spin rows) of inbox slot q: 16-byte planes [.][ns]
+// Shared-memory layouts in pieces of a warp's 32 sites (inbox: of 8 slots), so that
+// every plane lies at a compile-time offset from one address: with planes of T
+// sites each load had its own address arithmetic, a sixth of an MR step's
+// instructions.
+//
+// The site vectors rho and y: FP32 float4 [warp][6][32], FP64 double2 [warp][12][32].
 template <class C>
-__device__ __forceinline__ void half_load(const unsigned char* base, int ns, int q, cx<C> h0[3], cx<C> h1[3]) {
-    if constexpr (sizeof(C) == 4) {
-        const float4* p = reinterpret_cast<const float4*>(base) + q;
-        const float4 a = p[0], b = p[ns], c = p[2 * ns];
-        h0[0] = mk<C>(a.x, a.y), h0[1] = mk<C>(a.z, a.w), h0[2] = mk<C>(b.x, b.y);
-        h1[0] = mk<C>(b.z, b.w), h1[1] = mk<C>(c.x, c.y), h1[2] = mk<C>(c.z, c.w);
-    } else {
-        const double2* p = reinterpret_cast<const double2*>(base) + q;
+struct SiteVec {
+    static constexpr int kPlanes = sizeof(C) == 4 ? 6 : 12;
+    static constexpr int kWarp = kPlanes * 512;  // bytes of 32 sites
+    static __device__ __forceinline__ int at(int t) { return (t >> 5) * kWarp + (t & 31) * 16; }
+    static __device__ __forceinline__ void store(unsigned char* p, const cx<C> v[12]) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const double2 a = p[i * ns], b = p[(3 + i) * ns];
-            h0[i] = mk<C>(a.x, a.y);
-            h1[i] = mk<C>(b.x, b.y);
+        for (int q = 0; q < kPlanes; ++q)
+            if constexpr (sizeof(C) == 4)
+                *reinterpret_cast<float4*>(p + 512 * q) =
+                    make_float4(v[2 * q].re, v[2 * q].im, v[2 * q + 1].re, v[2 * q + 1].im);
+            else
+                *reinterpret_cast<double2*>(p + 512 * q) = make_double2(v[q].re, v[q].im);
+    }
+    static __device__ __forceinline__ void load(const unsigned char* p, cx<C> v[12]) {
+#pragma unroll
+        for (int q = 0; q < kPlanes; ++q)
+            if constexpr (sizeof(C) == 4) {
+                const float4 a = *reinterpret_cast<const float4*>(p + 512 * q);
+                v[2 * q] = mk<C>(a.x, a.y);
+                v[2 * q + 1] = mk<C>(a.z, a.w);
+            } else {
+                const double2 a = *reinterpret_cast<const double2*>(p + 512 * q);
+                v[q] = mk<C>(a.x, a.y);
+            }
+    }
+};
+
+// The links of a domain, per warp [4 directions] of
+//   P64      double2 [9][32]
+//   P32      float4 [4][32] (entries 2q, 2q + 1), float2 [32] (entry 8)
+//   P16/B16  uint4 [2][32] (entries 4q .. 4q + 3), uint32 [32] (entry 8)
+template <int PL>
+struct LinkWarp {
+    static constexpr int kEntry = PL == P64 ? 16 : PL == P32 ? 8 : 4;  // bytes of one complex entry
+    static constexpr int kMu = 9 * 32 * kEntry;                        // bytes of 32 sites' links in one direction
+    static constexpr int kWarp = 4 * kMu;
+    template <class C>
+    static __device__ __forceinline__ void load(const unsigned char* L, int mu, int t, cx<C> u[9]) {
+        const unsigned char* b = L + (t >> 5) * kWarp + mu * kMu;
+        const unsigned char* p = b + (t & 31) * 16;
+        if constexpr (PL == P64) {
+#pragma unroll
+            for (int c = 0; c < 9; ++c) {
+                const double2 v = *reinterpret_cast<const double2*>(p + 512 * c);
+                u[c] = mk<C>((C)v.x, (C)v.y);
+            }
+        } else if constexpr (PL == P32) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 v = *reinterpret_cast<const float4*>(p + 512 * q);
+                u[2 * q] = mk<C>((C)v.x, (C)v.y);
+                u[2 * q + 1] = mk<C>((C)v.z, (C)v.w);
+            }
+            const float2 v = *reinterpret_cast<const float2*>(b + 2048 + (t & 31) * 8);
+            u[8] = mk<C>((C)v.x, (C)v.y);
+        } else {
+            constexpr int bf = (PL == PB16);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint4 v = *reinterpret_cast<const uint4*>(p + 512 * q);
+                const float2 f0 = h2_to_f2(v.x, bf), f1 = h2_to_f2(v.y, bf), f2 = h2_to_f2(v.z, bf), f3 = h2_to_f2(v.w, bf);
+                u[4 * q] = mk<C>((C)f0.x, (C)f0.y);
+                u[4 * q + 1] = mk<C>((C)f1.x, (C)f1.y);
+                u[4 * q + 2] = mk<C>((C)f2.x, (C)f2.y);
+                u[4 * q + 3] = mk<C>((C)f3.x, (C)f3.y);
+            }
+            const float2 w = h2_to_f2(*reinterpret_cast<const uint32_t*>(b + 1024 + (t & 31) * 4), bf);
+            u[8] = mk<C>((C)w.x, (C)w.y);
         }
     }
-}
+    static __device__ __forceinline__ void pack(unsigned char* L, int t, const char* U, long long V, long long s) {
+        constexpr int N = PL == P64 ? 1 : PL == P32 ? 2 : 4;  // entries of a 16-byte word
+        for (int mu = 0; mu < 4; ++mu)
+            for (int c = 0; c < 9; ++c) {
+                unsigned char* b = L + (t >> 5) * kWarp + mu * kMu + (c / N) * 512;
+                unsigned char* to = (PL == P64 || c < 8) ? b + (t & 31) * 16 + (c % N) * kEntry : b + (t & 31) * kEntry;
+                const long long e = (long long)(mu * 9 + c) * V + s;
+                if constexpr (PL == P64)
+                    *reinterpret_cast<double2*>(to) = reinterpret_cast<const double2*>(U)[e];
+                else if constexpr (PL == P32)
+                    *reinterpret_cast<float2*>(to) = reinterpret_cast<const float2*>(U)[e];
+                else
+                    *reinterpret_cast<uint32_t*>(to) = reinterpret_cast<const uint32_t*>(U)[e];
+            }
+    }
+};
+
+// Half spinors (the upper two spin rows), in boxes of 8 slots: 16-byte words [3 or 6][8]
 template <class C>
-__device__ __forceinline__ void half_store(unsigned char* base, int ns, int q, const cx<C> h0[3], const cx<C> h1[3]) {
-    if constexpr (sizeof(C) == 4) {
-        float4* p = reinterpret_cast<float4*>(base) + q;
-        p[0] = make_float4(h0[0].re, h0[0].im, h0[1].re, h0[1].im);
-        p[ns] = make_float4(h0[2].re, h0[2].im, h1[0].re, h1[0].im);
-        p[2 * ns] = make_float4(h1[1].re, h1[1].im, h1[2].re, h1[2].im);
-    } else {
-        double2* p = reinterpret_cast<double2*>(base) + q;
+struct Half {
+    static constexpr int kWords = sizeof(C) == 4 ? 3 : 6;
+    static constexpr int kBox = kWords * 128;
+    static __host__ __device__ int bytes(int ns) { return (ns + 7) / 8 * kBox; }
+    static __device__ __forceinline__ int at(int q) { return (q >> 3) * kBox + (q & 7) * 16; }
+    static __device__ __forceinline__ void load(const unsigned char* p, cx<C> h0[3], cx<C> h1[3]) {
+        if constexpr (sizeof(C) == 4) {
+            const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 128),
+                         c = *reinterpret_cast<const float4*>(p + 256);
+            h0[0] = mk<C>(a.x, a.y), h0[1] = mk<C>(a.z, a.w), h0[2] = mk<C>(b.x, b.y);
+            h1[0] = mk<C>(b.z, b.w), h1[1] = mk<C>(c.x, c.y), h1[2] = mk<C>(c.z, c.w);
+        } else {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            p[i * ns] = make_double2(h0[i].re, h0[i].im);
-            p[(3 + i) * ns] = make_double2(h1[i].re, h1[i].im);
+            for (int i = 0; i < 3; ++i) {
+                const double2 a = *reinterpret_cast<const double2*>(p + 128 * i),
+                              b = *reinterpret_cast<const double2*>(p + 128 * (3 + i));
+                h0[i] = mk<C>(a.x, a.y);
+                h1[i] = mk<C>(b.x, b.y);
+            }
         }
     }
-}
+    static __device__ __forceinline__ void store(unsigned char* p, const cx<C> h0[3], const cx<C> h1[3]) {
+        if constexpr (sizeof(C) == 4) {
+            *reinterpret_cast<float4*>(p) = make_float4(h0[0].re, h0[0].im, h0[1].re, h0[1].im);
+            *reinterpret_cast<float4*>(p + 128) = make_float4(h0[2].re, h0[2].im, h1[0].re, h1[0].im);
+            *reinterpret_cast<float4*>(p + 256) = make_float4(h1[1].re, h1[1].im, h1[2].re, h1[2].im);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                *reinterpret_cast<double2*>(p + 128 * i) = make_double2(h0[i].re, h0[i].im);
+                *reinterpret_cast<double2*>(p + 128 * (3 + i)) = make_double2(h1[i].re, h1[i].im);
+            }
+        }
+    }
+};
 
 // what a face site sends: SIDE 0, its lower face: (1 + gamma_MU) y; SIDE 1,
 // its upper face: U^dagger (1 - gamma_MU) y
-template <int MU, class C, class LS>
-__device__ __forceinline__ void face_half(int side, const cx<C> y[12], const unsigned char* lsh, int T, int t,
-                                          cx<C> k0[3], cx<C> k1[3]) {
+template <int MU, class C, class LW>
+__device__ __forceinline__ void face_half(int side, const cx<C> y[12], const unsigned char* lsh, int t, cx<C> k0[3],
+                                          cx<C> k1[3]) {
     if (side == 0) {
-        project<MU, +1, C, true>(y, k0, k1);
+        project<MU, +1, C>(y, k0, k1);
     } else {
         cx<C> h0[3], h1[3], u[9];
-        project<MU, -1, C, true>(y, h0, h1);
-        LS::template load<C>(lsh, T, MU, t, u);
-        su3_mul<C, true, true>(u, h0, k0);
-        su3_mul<C, true, true>(u, h1, k1);
+        project<MU, -1, C>(y, h0, h1);
+        LW::template load<C>(lsh, MU, t, u);
+        su3_mul<C, true, kChain>(u, h0, k0);
+        su3_mul<C, true, kChain>(u, h1, k1);
+    }
+}
+
+// CTA-wide sums of three numbers, at most 8 warps: within a warp the three
+// are folded together (lanes end up with one number each), across warps every
+// lane adds one warp's numbers. red: [8][4].
+template <class C>
+__device__ __forceinline__ void cta_sum3(C& a, C& b, C& c, C* red) {
+    constexpr unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    // lanes 0-15 keep (a, b), lanes 16-31 (c, 0); then groups of 8 lanes a, b, c, 0
+    const C k0 = (h16 ? c : a) + __shfl_xor_sync(full, h16 ? a : c, 16);
+    const C k1 = (h16 ? C(0) : b) + __shfl_xor_sync(full, h16 ? b : C(0), 16);
+    C k = (h8 ? k1 : k0) + __shfl_xor_sync(full, h8 ? k0 : k1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(full, k, o);
+    if ((lane & 7) == 0) red[4 * (threadIdx.x >> 5) + (lane >> 3)] = k;
+    __syncthreads();
+    const int w = lane & 7;
+    const bool on = w < nw;
+    a = on ? red[4 * w] : C(0);
+    b = on ? red[4 * w + 1] : C(0);
+    c = on ? red[4 * w + 2] : C(0);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(full, a, o);
+        b += __shfl_xor_sync(full, b, o);
+        c += __shfl_xor_sync(full, c, o);
     }
 }
 
@@ -154,16 +284,16 @@ __device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target)
 template <int PS, int PL, class C, bool CLOV>
 __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(const __grid_constant__ SapArgs<C> a) {
     constexpr int CP = (sizeof(C) == 4) ? P32 : P64;  // layout of rho and xpart, storage of the clover term
-    constexpr int HB = 12 * (int)sizeof(C);           // bytes of a half spinor
-    typedef LinkSh<PL> LS;
+    typedef LinkWarp<PL> LW;
+    typedef SiteVec<C> SV;
+    typedef Half<C> HB;
     extern __shared__ __align__(16) unsigned char smem[];
     const Geom& g = a.g;
-    const int T = blockDim.x, ns = a.ns;
-    const int rbytes = max((int)sizeof(C) * 24 * T, HB * ns);
-    unsigned char* rsh = smem;                                    // inbox, then rho, then y
-    unsigned char* lsh = smem + rbytes;                           // links
-    C* red = reinterpret_cast<C*>(lsh + (size_t)LS::kBytes * T);  // [32][3]
-    unsigned long long* lbar = reinterpret_cast<unsigned long long*>(red + 96);
+    const int T = blockDim.x, ns = a.ns, hbytes = HB::bytes(ns);
+    unsigned char* rsh = smem;                                          // inbox, then rho, then y
+    unsigned char* lsh = smem + max(SV::kWarp * (T >> 5), hbytes);      // links
+    C* red = reinterpret_cast<C*>(lsh + LW::kWarp * (T >> 5));          // [8][4]
+    unsigned long long* lbar = reinterpret_cast<unsigned long long*>(red + 32);
 
     const int r = blockIdx.x % a.nrhs;
     const int e = blockIdx.x / a.nrhs;
@@ -188,7 +318,8 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
         lx[3] = q / g.b[2];
     }
     const int ls1 = g.b[0], ls2 = g.b[0] * g.b[1], ls3 = g.b[0] * g.b[1] * g.b[2];  // in-domain strides
-    const unsigned lbytes = (unsigned)LS::kBytes * (unsigned)T;
+    const unsigned lbytes = (unsigned)LW::kWarp * (unsigned)(T >> 5);
+    unsigned char* own = rsh + SV::at(tid);
     const unsigned char* limg = reinterpret_cast<const unsigned char*>(a.Uimg);
     const int dst1 = g.nb[0], dst2 = dst1 * g.nb[1], dst3 = dst2 * g.nb[2];
 
@@ -226,6 +357,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();  // the mbarrier is initialised before any thread waits on it
 
+    const C m2diag = -2 * a.diag;
     bool dead = false;
     for (int sw = a.s0; sw < a.s1; ++sw) {
         const bool first = sw < 2, last = sw >= a.nsweeps - 2;
@@ -255,8 +387,8 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
             __syncthreads();
         }
         if (sw > 0) {
-            const unsigned char* src = inb + (long long)dom * HB * ns;
-            for (int q = tid; q < HB / 16 * ns; q += T)
+            const unsigned char* src = inb + (long long)dom * hbytes;
+            for (int q = tid; q < hbytes / 16; q += T)
                 cp_async_word(reinterpret_cast<float4*>(rsh) + q, reinterpret_cast<const float4*>(src) + q);
             cp_async_wait();
         }
@@ -279,11 +411,11 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
                                             : mu == 2       ? (g.b[2] - 1) * ls2
                                                             : (g.b[3] - 1) * ls3);
                 cx<C> h0[3], h1[3], k0[3], k1[3], u[9];
-                half_load<C>(rsh, ns, q, h0, h1);
-                LS::template load<C>(lsh, T, mu, t, u);
-                su3_mul<C, false, true>(u, h0, k0);
-                su3_mul<C, false, true>(u, h1, k1);
-                half_store<C>(rsh, ns, q, k0, k1);
+                HB::load(rsh + HB::at(q), h0, h1);
+                LW::template load<C>(lsh, mu, t, u);
+                su3_mul<C, false, kChain>(u, h0, k0);
+                su3_mul<C, false, kChain>(u, h1, k1);
+                HB::store(rsh + HB::at(q), k0, k1);
             }
             __syncthreads();
             // ... then each site adds what enters through its faces
@@ -296,12 +428,12 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
     {                                                           \
         const int q = off + (FI);                               \
         if (lx[MU] == g.b[MU] - 1) {                            \
-            half_load<C>(rsh, ns, q, k0, k1);                   \
-            reconstruct<MU, +1, C, true>(k0, k1, acc);          \
+            HB::load(rsh + HB::at(q), k0, k1);                  \
+            reconstruct<MU, +1, C>(k0, k1, acc);                \
         }                                                       \
         if (lx[MU] == 0) {                                      \
-            half_load<C>(rsh, ns, ns / 2 + q, k0, k1);          \
-            reconstruct<MU, -1, C, true>(k0, k1, acc);          \
+            HB::load(rsh + HB::at(ns / 2 + q), k0, k1);         \
+            reconstruct<MU, -1, C>(k0, k1, acc);                \
         }                                                       \
         off += g.B / g.b[MU];                                   \
     }
@@ -319,28 +451,29 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
 #pragma unroll
         for (int c = 0; c < 12; ++c) y[c] = czero<C>();
 
-        // MR on D^l y = r^l out of shared memory
+        // MR on D^l y = r^l out of shared memory, with p = -2 D^l rho:
+        // beta = <p, rho> / <p, p>, y -= 2 beta rho, rho -= beta p
         for (int it = 0; it < a.nmr; ++it) {
-            rho_store<C>(rsh, T, tid, rho);
-            __syncthreads();
             cx<C> p[12];
+            SV::store(own, rho);
+#pragma unroll
+            for (int c = 0; c < 12; ++c) p[c] = m2diag * rho[c];
+            __syncthreads();
             C pr_re = 0, pr_im = 0, pp = 0;
             if (act) {
-                cx<C> acc[12], psi[12], u[9];
-#pragma unroll
-                for (int c = 0; c < 12; ++c) acc[c] = czero<C>();
+                cx<C> psi[12], u[9];
 #define SAP_LOC_HOPS(MU, LS_MU)                     \
     {                                               \
         if (lx[MU] + 1 < g.b[MU]) {                 \
-            rho_load<C>(rsh, T, tid + LS_MU, psi);  \
-            LS::template load<C>(lsh, T, MU, tid, u); \
-            hop<MU, +1, C, true>(psi, u, acc);      \
+            SV::load(rsh + SV::at(tid + LS_MU), psi); \
+            LW::template load<C>(lsh, MU, tid, u);  \
+            hop<MU, +1, C, kChain>(psi, u, p);      \
         }                                           \
         if (lx[MU] >= 1) {                          \
             const int tn = tid - LS_MU;             \
-            rho_load<C>(rsh, T, tn, psi);           \
-            LS::template load<C>(lsh, T, MU, tn, u); \
-            hop<MU, -1, C, true>(psi, u, acc);      \
+            SV::load(rsh + SV::at(tn), psi);        \
+            LW::template load<C>(lsh, MU, tn, u);   \
+            hop<MU, -1, C, kChain>(psi, u, p);      \
         }                                           \
     }
                 SAP_LOC_HOPS(0, 1)
@@ -351,35 +484,34 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
                 // the site's own rho is read back from shared memory (where the
                 // neighbours read it) rather than kept in registers over the hops:
                 // the 24 registers go to overlapping the hops' loads
-                rho_load<C>(rsh, T, tid, rho);
-                if constexpr (CLOV) clover_acc<CP, C>(a.clov, g.V, s, rho, acc, (C)-2);  // A rho as -2 A rho in acc
-                const C half = (C)0.5;
+                SV::load(own, rho);
+                if constexpr (CLOV) clover_acc<CP, C>(a.clov, g.V, s, rho, p, (C)-2);
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    p[c] = a.diag * rho[c] - half * acc[c];
-                    const cx<C> t = cmulc(p[c], rho[c]);
-                    pr_re += t.re;
-                    pr_im += t.im;
-                    pp += p[c].re * p[c].re + p[c].im * p[c].im;
+                    pr_re = fma(p[c].re, rho[c].re, pr_re);
+                    pr_im = fma(p[c].re, rho[c].im, pr_im);
+                    pp = fma(p[c].re, p[c].re, pp);
+                    pr_re = fma(p[c].im, rho[c].im, pr_re);
+                    pr_im = fma(-p[c].im, rho[c].re, pr_im);
+                    pp = fma(p[c].im, p[c].im, pp);
                 }
-            } else {
-#pragma unroll
-                for (int c = 0; c < 12; ++c) p[c] = czero<C>();
             }
-            block_sum3(pr_re, pr_im, pp, red);
+            cta_sum3(pr_re, pr_im, pp, red);
             if (pp > (C)0) {
-                const cx<C> alpha = mk<C>(pr_re / pp, pr_im / pp);
+                const C b_re = pr_re / pp, b_im = pr_im / pp, a_re = -2 * b_re, a_im = -2 * b_im;
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    y[c] = y[c] + alpha * rho[c];
-                    rho[c] = rho[c] - alpha * p[c];
+                    y[c].re = fma(-a_im, rho[c].im, fma(a_re, rho[c].re, y[c].re));
+                    y[c].im = fma(a_im, rho[c].re, fma(a_re, rho[c].im, y[c].im));
+                    rho[c].re = fma(b_im, p[c].im, fma(-b_re, p[c].re, rho[c].re));
+                    rho[c].im = fma(-b_im, p[c].re, fma(-b_re, p[c].im, rho[c].im));
                 }
             }
         }
 
         // the correction's half spinors to the neighbouring domains' inboxes
         if (sw + 1 < a.nsweeps) {
-            rho_store<C>(rsh, T, tid, y);
+            SV::store(own, y);
             __syncthreads();
             for (int q = tid; q < ns; q += T) {
                 const int side = q >= ns / 2 ? 1 : 0;
@@ -395,8 +527,8 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
         } else {                                                                             \
             to = D[MU] > 0 ? dom - DST : dom + (g.nb[MU] - 1) * DST;                         \
         }                                                                                    \
-        rho_load<C>(rsh, T, t, yy);                                                          \
-        face_half<MU, C, LS>(side, yy, lsh, T, t, k0, k1);                                   \
+        SV::load(rsh + SV::at(t), yy);                                                       \
+        face_half<MU, C, LW>(side, yy, lsh, t, k0, k1);                                      \
     }
                 if (mu == 0)
                     SAP_SEND(0, 1, 1)
@@ -407,7 +539,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
                 else
                     SAP_SEND(3, ls3, dst3)
 #undef SAP_SEND
-                half_store<C>(inb + to * HB * ns, ns, q, k0, k1);
+                HB::store(inb + to * hbytes + HB::at(q), k0, k1);
             }
         }
         const long long sc = s;  // this sweep's site
@@ -442,6 +574,40 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
             a.bar[r] = 0u;
             *ex = 0u;
         }
+    }
+}
+
+// the links of domain blockIdx.x (both colours) as LinkWarp keeps them in shared memory
+template <int PL>
+__global__ void warp_image_kernel(Geom g, const char* __restrict__ U, char* __restrict__ img) {
+    const int t = threadIdx.x;
+    if (t >= g.B) return;
+    int D[4], q = blockIdx.x;
+    D[0] = q % g.nb[0];
+    q /= g.nb[0];
+    D[1] = q % g.nb[1];
+    q /= g.nb[1];
+    D[2] = q % g.nb[2];
+    D[3] = q / g.nb[2];
+    int xg[4], r = t;
+    for (int j = 0; j < 3; ++j) {
+        xg[j] = D[j] * g.b[j] + r % g.b[j];
+        r /= g.b[j];
+    }
+    xg[3] = D[3] * g.b[3] + r;
+    LinkWarp<PL>::pack(reinterpret_cast<unsigned char*>(img) + (size_t)blockIdx.x * LinkWarp<PL>::kWarp * (blockDim.x >> 5),
+                       t, U, g.V, site_index(g, xg));
+}
+
+// faces[q]: lower-face site | mu << 10 of inbox slot q (and of its mirror q + ns / 2)
+__global__ void faces_kernel(Geom g, unsigned short* faces) {
+    int ls = 1, off = 0;
+    for (int mu = 0; mu < 4; ++mu) {
+        for (int t = threadIdx.x; t < g.B; t += blockDim.x)
+            if ((t / ls) % g.b[mu] == 0)  // the slots run over the other three coordinates in order
+                faces[off + t % ls + ls * (t / (ls * g.b[mu]))] = (unsigned short)(t | (mu << 10));
+        off += g.B / g.b[mu];
+        ls *= g.b[mu];
     }
 }
 
@@ -533,25 +699,46 @@ int sap_inbox_slots(const Geom& g) {
 
 int sap_apply_smem(int pspin, int plink, const Geom& g) {
     const int c = (pspin == P64) ? 8 : 4, T = sap_threads(g, 0);
-    const int body = std::max(c * 24 * T, c * 12 * sap_inbox_slots(g));
-    return body + (int)(sap_link_image_bytes(plink, g, T) / g.ndom) + c * 96 + 16;
+    const int body = std::max(c * 24 * T, (int)(sap_inbox_bytes(pspin, g) / g.ndom));
+    return body + (int)(sap_link_image_bytes(plink, g, T) / g.ndom) + c * 32 + 16;
 }
 
 // Domains of at most 256 sites whose inbox is no larger than a double-precision
 // field (the scratch that a solve has at hand) and fits in shared memory.
 bool sap_apply_fits(int prec, const Geom& g) {
-    const long long c = (prec == P64) ? 8 : 4;
-    return g.B <= 256 && 12 * c * sap_inbox_slots(g) <= 192LL * g.B && sap_apply_smem(prec, prec, g) <= 227 * 1024;
+    return g.B <= 256 && sap_inbox_bytes(prec, g) <= 192 * (size_t)g.V && sap_apply_smem(prec, prec, g) <= 227 * 1024;
 }
 
-void sap_faces(const Geom& g, std::vector<unsigned short>* out) {
-    out->clear();
-    int ls = 1;
-    for (int mu = 0; mu < 4; ++mu) {
-        for (int t = 0; t < g.B; ++t)
-            if ((t / ls) % g.b[mu] == 0) out->push_back((unsigned short)(t | (mu << 10)));
-        ls *= g.b[mu];
-    }
+size_t sap_state_bytes(int prec, const Geom& g) {
+    const bool half = (prec == P16 || prec == PB16);
+    return (size_t)spinor_bytes(prec == P64 ? P64 : P32, g.V) * (half ? 2 : 1);
+}
+
+size_t sap_inbox_bytes(int prec, const Geom& g) {
+    const int ns = sap_inbox_slots(g);
+    return (size_t)g.ndom * (prec == P64 ? Half<double>::bytes(ns) : Half<float>::bytes(ns));
+}
+
+int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st) {
+    const int T = sap_threads(g, 0);
+    if (T != g.B) DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(prec, g, T), st));  // rows of idle threads
+    const unsigned nb = (unsigned)g.ndom;
+    if (prec == P64)
+        warp_image_kernel<P64><<<nb, T, 0, st>>>(g, U, img);
+    else if (prec == P32)
+        warp_image_kernel<P32><<<nb, T, 0, st>>>(g, U, img);
+    else if (prec == P16)
+        warp_image_kernel<P16><<<nb, T, 0, st>>>(g, U, img);
+    else
+        warp_image_kernel<PB16><<<nb, T, 0, st>>>(g, U, img);
+    DW_LAUNCH_CHECK();
+    return DW_OK;
+}
+
+int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st) {
+    faces_kernel<<<1, 256, 0, st>>>(g, faces);
+    DW_LAUNCH_CHECK();
+    return DW_OK;
 }
 
 int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab,
