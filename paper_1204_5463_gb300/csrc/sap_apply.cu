@@ -25,13 +25,13 @@
 // (5.3 us of a 22 us sweep), and a launch per sweep costs 8-9 us between the
 // sweeps of 256 domains. Here the residual takes 1.8 us, and the sends 1.2 us.
 // Measured against one launch of sap_sweep_kernel per sweep (5 cycles x 4 MR
-// steps unless stated): 8^3 x 16, 2 rhs served on 4 streams 38.2 -> 29.4 ms a
-// burst; 12^3 x 18 in 3^4 domains, 3 BF16 rhs (4 x 5) 341 -> 289 us; 24^3 x 48,
-// 12 FP16 rhs 14.91 -> 12.87 ms; 16^3 x 32 FP32 342 -> 314 us, with the clover
-// term (8 x 5) 766 -> 641 us. Four fifths of that are the MR steps: 4800 cycles
-// a step for the one domain of an SM, 7700 for two, of which the shared-memory
-// pipe is busy 5900 (367 wavefronts a warp and step); paired, scalar and mixed
-// forms of the hop's FP32 arithmetic are all within 2% of one another.
+// steps unless stated): 8^3 x 16, 2 rhs served on 4 streams 38.2 -> 28.8 ms a
+// burst; 12^3 x 18 in 3^4 domains, 3 BF16 rhs (4 x 5) 341 -> 279 us; 24^3 x 48,
+// 12 FP16 rhs 14.91 -> 12.48 ms; 16^3 x 32 FP32 342 -> 302 us, with the clover
+// term (8 x 5) 766 -> 630 us. Four fifths of that are the MR steps, bound by the
+// latency of shared memory at the 16 warps that 128 registers allow, with its
+// pipe busy three quarters of the time; paired, scalar and mixed forms of the
+// hop's FP32 arithmetic are within 2% of one another.
 #include <map>
 #include <mutex>
 
@@ -233,6 +233,40 @@ __device__ __forceinline__ void face_half(int side, const cx<C> y[12], const uns
         su3_mul<C, true, kChain>(u, h0, k0);
         su3_mul<C, true, kChain>(u, h1, k1);
     }
+}
+
+// acc += m times the spin rows rebuilt from k0, k1 (m = 0: a neighbour outside the domain)
+template <int MU, int SIGN, class C>
+__device__ __forceinline__ void reconstruct_if(C m, const cx<C> k0[3], const cx<C> k1[3], cx<C> acc[12]) {
+    const C s = SIGN > 0 ? m : -m;
+    auto add = [](cx<C>& to, C w, cx<C> k) { to = mk<C>(fma(w, k.re, to.re), fma(w, k.im, to.im)); };
+    auto addi = [](cx<C>& to, C w, cx<C> k) { to = mk<C>(fma(-w, k.im, to.re), fma(w, k.re, to.im)); };  // + i w k
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        add(acc[c], m, k0[c]);
+        add(acc[3 + c], m, k1[c]);
+        if constexpr (MU == 0) {
+            addi(acc[6 + c], s, k1[c]);
+            addi(acc[9 + c], s, k0[c]);
+        } else if constexpr (MU == 1) {
+            add(acc[6 + c], s, k1[c]);
+            add(acc[9 + c], -s, k0[c]);
+        } else if constexpr (MU == 2) {
+            addi(acc[6 + c], s, k0[c]);
+            addi(acc[9 + c], -s, k1[c]);
+        } else {
+            add(acc[6 + c], s, k0[c]);
+            add(acc[9 + c], s, k1[c]);
+        }
+    }
+}
+template <int MU, int SIGN, class C>
+__device__ __forceinline__ void hop_if(bool in, const cx<C> psi[12], const cx<C> u[9], cx<C> acc[12]) {
+    cx<C> h0[3], h1[3], k0[3], k1[3];
+    project<MU, SIGN, C>(psi, h0, h1);
+    su3_mul<C, (SIGN < 0), kChain>(u, h0, k0);
+    su3_mul<C, (SIGN < 0), kChain>(u, h1, k1);
+    reconstruct_if<MU, SIGN, C>(in ? C(1) : C(0), k0, k1, acc);
 }
 
 // CTA-wide sums of three numbers, at most 8 warps: within a warp the three
@@ -462,25 +496,35 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
             C pr_re = 0, pr_im = 0, pp = 0;
             if (act) {
                 cx<C> psi[12], u[9];
-#define SAP_LOC_HOPS(MU, LS_MU)                     \
-    {                                               \
-        if (lx[MU] + 1 < g.b[MU]) {                 \
-            SV::load(rsh + SV::at(tid + LS_MU), psi); \
-            LW::template load<C>(lsh, MU, tid, u);  \
-            hop<MU, +1, C, kChain>(psi, u, p);      \
-        }                                           \
-        if (lx[MU] >= 1) {                          \
-            const int tn = tid - LS_MU;             \
-            SV::load(rsh + SV::at(tn), psi);        \
-            LW::template load<C>(lsh, MU, tn, u);   \
-            hop<MU, -1, C, kChain>(psi, u, p);      \
-        }                                           \
+                // directions 0 to 2 without branches, so that the loads of one hop
+                // overlap the arithmetic of another (a neighbour outside the domain
+                // is the site itself, with weight 0); direction 3, whose hops whole
+                // warps skip at the domain's ends, with them
+#define SAP_ALL_HOPS(MU, LS_MU)                          \
+    {                                                    \
+        const bool up = lx[MU] + 1 < g.b[MU], dn = lx[MU] >= 1; \
+        const int tu = up ? tid + LS_MU : tid, td = dn ? tid - LS_MU : tid; \
+        SV::load(rsh + SV::at(tu), psi);                 \
+        LW::template load<C>(lsh, MU, tid, u);           \
+        hop_if<MU, +1, C>(up, psi, u, p);                \
+        SV::load(rsh + SV::at(td), psi);                 \
+        LW::template load<C>(lsh, MU, td, u);            \
+        hop_if<MU, -1, C>(dn, psi, u, p);                \
     }
-                SAP_LOC_HOPS(0, 1)
-                SAP_LOC_HOPS(1, ls1)
-                SAP_LOC_HOPS(2, ls2)
-                SAP_LOC_HOPS(3, ls3)
-#undef SAP_LOC_HOPS
+                SAP_ALL_HOPS(0, 1)
+                SAP_ALL_HOPS(1, ls1)
+                SAP_ALL_HOPS(2, ls2)
+#undef SAP_ALL_HOPS
+                if (lx[3] + 1 < g.b[3]) {
+                    SV::load(rsh + SV::at(tid + ls3), psi);
+                    LW::template load<C>(lsh, 3, tid, u);
+                    hop<3, +1, C, kChain>(psi, u, p);
+                }
+                if (lx[3] >= 1) {
+                    SV::load(rsh + SV::at(tid - ls3), psi);
+                    LW::template load<C>(lsh, 3, tid - ls3, u);
+                    hop<3, -1, C, kChain>(psi, u, p);
+                }
                 // the site's own rho is read back from shared memory (where the
                 // neighbours read it) rather than kept in registers over the hops:
                 // the 24 registers go to overlapping the hops' loads
