@@ -231,6 +231,30 @@ __device__ __forceinline__ df df_warp_sum(df a) {
 }
 #endif
 
+#ifdef __CUDACC__
+// FP64 <-> FP32 by integer operations, the same bits as the conversion
+// instructions, which run at the FP64 pipe's rate (1/64 of FP32 on this part:
+// 24 of them a site bound every copy between the caller's FP64 layout and the
+// FP32-class formats at 2.8 TB/s). Each takes numbers whose result is a normal
+// FP32 number or zero and reports whether the argument was one; the
+// caller converts the others with the instruction.
+__device__ __forceinline__ float narrow(double x, bool& ok) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), a = hi & 0x7fffffffu;
+    const bool zero = (a | lo) == 0u;
+    ok = ok && (zero || a - 0x38100000u < 0x0fe00000u);  // 0 or 2^-126 <= |x| < 2^128
+    // the exponent rebiased, 23 bits of the significand, then round to nearest even
+    const unsigned b = __funnelshift_l(lo, a - 0x38000000u, 3);
+    const unsigned up = ((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29;
+    return __uint_as_float((zero ? 0u : b + up) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double widen(float x, bool& ok) {
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu, e = a >> 23;
+    ok = ok && (a == 0u || e - 1u < 254u);
+    const unsigned hi = a == 0u ? u : ((a >> 3) + 0x38000000u) | (u & 0x80000000u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+#endif
+
 template <int P>
 struct real_of {
     typedef float type;
