@@ -344,21 +344,19 @@ int dw_apply(dw_ctx* ctx, const double* in, double* out, dw_prec prec, int nrhs)
     const char* U;
     if ((rc = gauge_for(ctx, prec, &U))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
-    if ((rc = ctx->work_out.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = launch_to_internal(prec, in, ctx->work_in.as<char>(), V, nrhs, ctx->stream))) return rc;
     {
-        // algorithmic bytes: every field once, the links once for all
+        // algorithmic bytes: every field once (the input in storage precision,
+        // the output in the caller's FP64 layout), the links once for all
         // right-hand sides of the launch (its CTAs for one block of sites and
         // the different rhs run next to each other, so L2 serves the re-reads)
         const double link_reads = 1.0;
         ProfScope ps(&ctx->prof, prec == DW_F64 ? "dw_f64" : prec == DW_F32 ? "dw_f32" : "dw_f16",
-                     (double)nrhs * 2.0 * fb + link_reads * link_bytes(prec, V));
-        FieldRef fi{ctx->work_in.as<char>(), fb, 0, 0}, fo{ctx->work_out.as<char>(), fb, 0, 0};
-        if ((rc = launch_dw(prec, prec, prec, ctx->g, ctx->m0, fi, fo, U, nullptr, nrhs, nullptr, ctx->stream,
-                            ctx->clover())))
+                     (double)nrhs * (fb + 192.0 * V) + link_reads * link_bytes(prec, V));
+        if ((rc = launch_dw_out(prec, ctx->g, ctx->m0, ctx->work_in.as<char>(), out, U, nrhs, ctx->stream,
+                                ctx->clover())))
             return rc;
     }
-    if ((rc = launch_from_internal(prec, ctx->work_out.as<char>(), out, V, nrhs, ctx->stream))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return DW_OK;
 }

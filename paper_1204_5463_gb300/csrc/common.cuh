@@ -399,6 +399,24 @@ __device__ __forceinline__ void store_spinor(char* base, long long V, long long 
     }
 }
 
+// v as store_spinor<P> followed by load_spinor<P> returns it
+template <int P, class C>
+__device__ __forceinline__ void round_spinor(cx<C> v[12]) {
+    if constexpr (P == P16 || P == PB16) {
+        constexpr int bf = (P == PB16);
+        float mx = 0.f;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) mx = fmaxf(mx, fmaxf(fabsf((float)v[c].re), fabsf((float)v[c].im)));
+        const float sc = (mx > 0.f) ? mx : 1.f;
+        const float inv = 1.f / sc;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const float2 h = h2_to_f2(f2_to_h2((float)v[c].re * inv, (float)v[c].im * inv, bf), bf);
+            v[c] = mk<C>((C)(sc * h.x), (C)(sc * h.y));
+        }
+    }
+}
+
 // link U_{s,mu} (3x3, row-major) in compute type C
 template <int P, class C, bool G = true>
 __device__ __forceinline__ void load_link(const char* base, long long V, int mu, long long s, cx<C> u[9]) {
@@ -627,6 +645,50 @@ __device__ __forceinline__ void hop(const cx<C> psi[12], const cx<C> u[9], cx<C>
     su3_mul<C, (SIGN < 0), PACK>(u, h0, k0);
     su3_mul<C, (SIGN < 0), PACK>(u, h1, k1);
     reconstruct<MU, SIGN, C, PACK>(k0, k1, acc);
+}
+
+// Both hops of direction MU for FP64 arithmetic, whose pipe bounds the stencil: the
+// link products are FMA chains, the forward one started from the backward one's
+// result, so that the sum of both costs no addition, and their difference one:
+// 204 instead of 264 FP64 instructions a direction. FIRST: acc holds nothing yet.
+template <int MU, bool FIRST>
+__device__ __forceinline__ void hop_pair(const cx<double> pf[12], const cx<double> uf[9], const cx<double> pb[12],
+                                         const cx<double> ub[9], cx<double> acc[12]) {
+    cx<double> f[2][3], b[2][3], kb[2][3];
+    project<MU, +1, double>(pf, f[0], f[1]);
+    project<MU, -1, double>(pb, b[0], b[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        su3_mul<double, true, 2>(ub, b[q], kb[q]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double re = kb[q][a].re, im = kb[q][a].im;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const cx<double> w = uf[3 * a + c];
+                re = fma(w.re, f[q][c].re, re);
+                im = fma(w.re, f[q][c].im, im);
+                re = fma(-w.im, f[q][c].im, re);
+                im = fma(w.im, f[q][c].re, im);
+            }
+            const cx<double> sum = mk<double>(re, im);
+            const cx<double> dif = mk<double>(fma(-2.0, kb[q][a].re, re), fma(-2.0, kb[q][a].im, im));
+            // lower row (common.cuh, reconstruct): the row and phase of k_q
+            constexpr bool cross = MU < 2;  // k0 feeds spin 3, k1 spin 2
+            const int row = 3 * ((q == 0) == cross ? 3 : 2) + a;
+            cx<double> low;
+            if (MU == 0)
+                low = ti(dif);
+            else if (MU == 1)
+                low = q == 0 ? mk<double>(-dif.re, -dif.im) : dif;
+            else if (MU == 2)
+                low = q == 0 ? ti(dif) : tmi(dif);
+            else
+                low = dif;
+            acc[3 * q + a] = FIRST ? sum : acc[3 * q + a] + sum;
+            acc[row] = FIRST ? low : acc[row] + low;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------

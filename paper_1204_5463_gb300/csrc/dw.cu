@@ -178,20 +178,34 @@ constexpr int dw_min_blocks() {
     return sizeof(C) != 4 ? 1 : (PI == P32 && PO == P32) ? 3 : (PI == P32) ? 4 : (PO == PI) ? 2 : 3;
 }
 
+// D at one site, diag psi - 1/2 hops (the clover term included), or b minus
+// that with b the field sub in format PO
 template <int PI, int PO, int PL, class C, bool SUB, bool CLOV>
-__global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
-    dw_kernel(Geom g, C diag, FieldRef in, FieldRef out, const char* U, const int* jtab, int nrhs, FieldRef sub,
-              const char* clov) {
-    const int r = blockIdx.x % nrhs;
-    const long long s = (blockIdx.x / nrhs) * (long long)blockDim.x + threadIdx.x;
-    if (s >= g.V || !rhs_active(jtab, r)) return;
-    const char* pin = field_ptr(in, jtab, r);
+__device__ __forceinline__ void dw_site(const Geom& g, C diag, const char* pin, const char* sub, const char* U,
+                                        const char* clov, long long s, cx<C> res[12]) {
     int x[4];
     site_coords(g, s, x);
-    cx<C> acc[12];
+    cx<C> acc[12], psi[12];
+    if constexpr (sizeof(C) == 8 && std::is_same<C, double>::value) {
+        cx<C> pb[12], u[9], ub[9];
+#define DW_PAIR(MU)                                                     \
+    {                                                                   \
+        const long long sm = neighbour(g, s, x, MU, -1);                \
+        load_spinor<PI, C>(pin, g.V, neighbour(g, s, x, MU, +1), psi);  \
+        load_link<PL, C>(U, g.V, MU, s, u);                             \
+        load_spinor<PI, C>(pin, g.V, sm, pb);                           \
+        load_link<PL, C>(U, g.V, MU, sm, ub);                           \
+        hop_pair<MU, MU == 0>(psi, u, pb, ub, acc);                     \
+    }
+        DW_PAIR(0)
+        DW_PAIR(1)
+        DW_PAIR(2)
+        DW_PAIR(3)
+#undef DW_PAIR
+    } else {
+        cx<C> u[9];
 #pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = czero<C>();
-    cx<C> psi[12], u[9];
+        for (int c = 0; c < 12; ++c) acc[c] = czero<C>();
 #define DW_HOPS(MU)                                                     \
     {                                                                   \
         const long long sp = neighbour(g, s, x, MU, +1);                \
@@ -203,26 +217,92 @@ __global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
         load_link<PL, C>(U, g.V, MU, sm, u);                            \
         hop<MU, -1, C>(psi, u, acc);                                    \
     }
-    DW_HOPS(0)
-    DW_HOPS(1)
-    DW_HOPS(2)
-    DW_HOPS(3)
+        DW_HOPS(0)
+        DW_HOPS(1)
+        DW_HOPS(2)
+        DW_HOPS(3)
 #undef DW_HOPS
+    }
     load_spinor<PI, C>(pin, g.V, s, psi);
     // clover term A psi_n, folded into the accumulator as -2 A psi_n
     if constexpr (CLOV) clover_acc<(sizeof(C) == 4) ? P32 : P64, C>(clov, g.V, s, psi, acc, C(-2.0f));
     const C half = C(0.5f);
-    cx<C> res[12];
     if constexpr (SUB) {
         cx<C> b[12];
-        load_spinor<PO, C>(field_ptr(sub, jtab, r), g.V, s, b);
+        load_spinor<PO, C>(sub, g.V, s, b);
 #pragma unroll
         for (int c = 0; c < 12; ++c) res[c] = b[c] - (diag * psi[c] - half * acc[c]);
     } else {
 #pragma unroll
         for (int c = 0; c < 12; ++c) res[c] = diag * psi[c] - half * acc[c];
     }
+}
+
+template <int PI, int PO, int PL, class C, bool SUB, bool CLOV>
+__global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
+    dw_kernel(Geom g, C diag, FieldRef in, FieldRef out, const char* U, const int* jtab, int nrhs, FieldRef sub,
+              const char* clov) {
+    const int r = blockIdx.x % nrhs;
+    const long long s = (blockIdx.x / nrhs) * (long long)blockDim.x + threadIdx.x;
+    if (s >= g.V || !rhs_active(jtab, r)) return;
+    cx<C> res[12];
+    dw_site<PI, PO, PL, C, SUB, CLOV>(g, diag, field_ptr(in, jtab, r), SUB ? field_ptr(sub, jtab, r) : nullptr, U, clov, s,
+                                      res);
     store_spinor<PO, C>(field_ptr(out, jtab, r), g.V, s, res);
+}
+
+// D with the result rounded to storage format P and written in the caller's
+// FP64 layout: what a stencil in P and a conversion back would give, without
+// the result's way through memory in between. A warp hands its 32 sites over
+// through shared memory, four of the twelve components at a time, so that it
+// writes 64 contiguous bytes of each site and the tile stays small beside L1,
+// on which the stencil lives. Stencil and conversion apart and together, 24^3 x
+// 48: FP32 one field 64 + 32 -> 81 us (HBM and latency), twelve FP16 fields 565
+// + 280 -> 790 us (instructions: 24 conversions and 24 scalings of every
+// neighbour); FP64 at 16^3 x 32 318 + 10 -> 232 us with hop_pair (the FP64 pipe:
+// 840 instructions a site take 190 us).
+template <int P, class C, bool CLOV>
+__global__ void __launch_bounds__(kThreads, dw_min_blocks<P, P, P, C>())
+    dw_out_kernel(Geom g, C diag, const char* in, long long in_rs, double* canon, const char* U, int nrhs,
+                  const char* clov) {
+    __shared__ __align__(16) double2 tiles[kThreads / 32][32 * 5];
+    const int r = blockIdx.x % nrhs, lane = threadIdx.x & 31;
+    const long long s0 = (blockIdx.x / nrhs) * (long long)blockDim.x + (threadIdx.x & ~31), s = s0 + lane;
+    if (s0 >= g.V) return;  // the whole warp
+    cx<C> res[12];
+    if (s < g.V) {
+        dw_site<P, P, P, C, false, CLOV>(g, diag, in + r * in_rs, nullptr, U, clov, s, res);
+        round_spinor<P, C>(res);
+    } else {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) res[c] = czero<C>();
+    }
+    double2* tile = tiles[threadIdx.x >> 5];
+    double2* dst = reinterpret_cast<double2*>(canon) + ((long long)r * g.V + s0) * 12;
+    const int n = (int)min(32LL, g.V - s0);
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+        bool done = sizeof(C) == 4;
+        if constexpr (sizeof(C) == 4) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double re = widen(res[4 * h + c].re, done), im = widen(res[4 * h + c].im, done);
+                tile[5 * lane + c] = make_double2(re, im);
+            }
+        }
+        if (!done) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                tile[5 * lane + c] = make_double2((double)res[4 * h + c].re, (double)res[4 * h + c].im);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = 8 * j + (lane >> 2);  // site
+            if (q < n) dst[12 * q + 4 * h + (lane & 3)] = tile[5 * q + (lane & 3)];
+        }
+        __syncwarp();
+    }
 }
 
 dim3 site_grid(long long V, int nrhs) { return dim3((unsigned)((V + kThreads - 1) / kThreads), nrhs); }
@@ -361,6 +441,29 @@ int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, co
     return fail(DW_EINVAL, "unsupported conversion");
 }
 
+int launch_dw_out(int prec, const Geom& g, double m0, const char* in, double* canon, const char* U, int nrhs,
+                  cudaStream_t st, const ClovRef* cl) {
+    const unsigned nb = (unsigned)((g.V + kThreads - 1) / kThreads) * (unsigned)nrhs;
+    const long long rs = spinor_bytes(prec, g.V);
+    const double d = 4.0 + m0;
+#define DWO(P, C)                                                                                                 \
+    if (prec == P) {                                                                                              \
+        const char* A = cl ? ((sizeof(C) == 4) ? cl->a32 : cl->a64) : nullptr;                                    \
+        if (cl)                                                                                                   \
+            dw_out_kernel<P, C, true><<<nb, kThreads, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);               \
+        else                                                                                                      \
+            dw_out_kernel<P, C, false><<<nb, kThreads, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);              \
+        DW_LAUNCH_CHECK();                                                                                        \
+        return DW_OK;                                                                                             \
+    }
+    DWO(P64, double)
+    DWO(P32, float)
+    DWO(P16, float)
+    DWO(PB16, float)
+#undef DWO
+    return fail(DW_EINVAL, "bad precision");
+}
+
 int launch_dw(int pin, int pout, int plink, const Geom& g, double m0, FieldRef in, FieldRef out, const char* U,
               const int* jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl) {
     // Supported combinations: uniform precision (the stencil as an operator),
@@ -369,8 +472,6 @@ int launch_dw(int pin, int pout, int plink, const Geom& g, double m0, FieldRef i
     if (pin == A && pout == B && plink == L) return dw_dispatch_sub<A, B, L, C>(g, m0, in, out, U, jtab, nrhs, sub, cl, st);
     DWC(P64, P64, P64, double)
     DWC(P32, P32, P32, float)
-    DWC(P16, P16, P16, float)
-    DWC(PB16, PB16, PB16, float)
     DWC(P16, P32, P32, float)
     DWC(PB16, P32, P32, float)
     DWC(P32, P64, P32, float)

@@ -172,6 +172,9 @@ int launch_link_convert(int prec, const char* U64, char* out, long long V, cudaS
 // with cl, D includes the clover term
 int launch_dw(int pin, int pout, int plink, const Geom& g, double m0, FieldRef in, FieldRef out, const char* U,
               const int* jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl = nullptr);
+// out (caller's FP64 layout, nrhs fields) = D in, all in storage precision prec (P64, P32, P16, PB16)
+int launch_dw_out(int prec, const Geom& g, double m0, const char* in, double* out, const char* U, int nrhs,
+                  cudaStream_t st, const ClovRef* cl = nullptr);
 // ----- clover.cu -----------------------------------------------------------
 int launch_clover_compute(const Geom& g, const char* U64, double csw, double* A64, float4* A32, cudaStream_t st);
 

@@ -1,5 +1,5 @@
 // dw_apply_f32_noalloc: the FP32 path of dw_apply (convert the input to the
-// internal FP32 layout, apply D, convert back) for callers that must not
+// internal FP32 layout, apply D, widen the result) for callers that must not
 // allocate device memory -- code running inside a pre-reserved memory pool,
 // under an allocator that forbids cudaMalloc, or in a process whose memory
 // budget is fixed at start-up. The internal-layout copies of the links and of
@@ -66,13 +66,9 @@ extern "C" int dw_apply_f32_noalloc(const int* dims, double m0, const double* U,
     const long long V = g.V;
     char* links = base;                               // 288 V
     char* fin = base + link_bytes(P32, kNoAllocMaxSites);   // 96 V
-    char* fout = fin + spinor_bytes(P32, kNoAllocMaxSites);  // 96 V
     if ((rc = launch_gauge_convert(P32, U, links, V, st))) return rc;
     if ((rc = launch_to_internal(P32, in, fin, V, 1, st))) return rc;
-    const long long fb = spinor_bytes(P32, V);
-    FieldRef fi{fin, fb, 0, 0}, fo{fout, fb, 0, 0};
-    if ((rc = launch_dw(P32, P32, P32, g, m0, fi, fo, links, nullptr, 1, nullptr, st))) return rc;
-    if ((rc = launch_from_internal(P32, fout, out, V, 1, st))) return rc;
+    if ((rc = launch_dw_out(P32, g, m0, fin, out, links, 1, st))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(st));
     return DW_OK;
 }
