@@ -190,39 +190,75 @@ struct Elem<PDF> {
 // coalesced; the warp reductions happen once per CTA at the end.
 constexpr int kDotG = 8;       // basis vectors per CTA
 constexpr int kDotStages = 3;  // elements in flight per thread
+constexpr int kMaxGroups = kDotCounters;
+static_assert(kMaxGroups * kDotG >= kMaxV, "a counter per group");
 
 template <int VP>
 constexpr size_t multidot_smem() {
     return (size_t)kDotStages * (kDotG + 1) * kT * sizeof(typename Elem<VP>::T);
 }
 
-// The last CTA of a launch (per rhs) to finish sums the partial rows:
-// fin[i] = sum_b part[b][i], each row lane-strided over b and then a fixed
-// shuffle tree, the order of the separate finalize kernel (so the result does
-// not depend on which CTA is last). Every CTA fences its partial writes and
-// counts itself in; the last one reads the rows through L2 and resets the
-// counter for the next launch on the stream.
-__device__ __forceinline__ void last_cta_sum(const double2* part, int nrow, int NP, unsigned* cnt, double2* fin) {
+// CTA-wide sum of one FP64 number per thread, returned to warp 0. The FP64 pipe
+// takes 16 cycles for a warp's addition, so each lane of one warp adds 8
+// numbers before the shuffles: 13 warp additions instead of 48.
+__device__ __forceinline__ double cta_sum(double a, double* sh) {
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int q = 0; q < kT / 32; ++q) s += sh[threadIdx.x + 32 * q];
+        s = warp_sum(s);
+    }
+    return s;
+}
+
+// Every CTA fences its partial sums and counts itself in; true for the last of
+// the n CTAs that share cnt, which may then read them through L2 and has set
+// the counter back to zero for the next launch on the stream.
+__device__ __forceinline__ bool last_cta(unsigned* cnt, unsigned n) {
     __shared__ unsigned is_last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(cnt, 1u) == gridDim.x - 1);
+    if (threadIdx.x == 0) {
+        is_last = (atomicAdd(cnt, 1u) == n - 1);
+        if (is_last) *cnt = 0u;
+    }
     __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < NP; i += nw) {
-        double2 s = make_double2(0.0, 0.0);
-        for (int b = lane; b < nrow; b += 32) {
+    if (is_last) __threadfence();
+    return is_last;
+}
+
+// fin[i] = sum_b part[b][i] for the G <= 8 rows of one group: thread t adds the
+// slots t / 8, t / 8 + 32, ... of row t % 8 (128 contiguous bytes of a slot), then
+// a fixed order over threads and warps, so that the result does not depend on
+// which CTA comes last. sh: 2 * kT doubles.
+__device__ __forceinline__ void group_sum(const double2* part, int nslots, int NP, int G, double2* fin, double* sh) {
+    const int i = threadIdx.x & 7, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double2 s = make_double2(0.0, 0.0);
+    if (i < G)
+        for (int b = threadIdx.x >> 3; b < nslots; b += kT / 8) {
             const double2 t = __ldcg(part + (long long)b * NP + i);
             s.x += t.x;
             s.y += t.y;
         }
-        s.x = warp_sum(s.x);
-        s.y = warp_sum(s.y);
-        if (lane == 0) fin[i] = s;
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
     }
-    if (threadIdx.x == 0) *cnt = 0u;
+    double2* w = reinterpret_cast<double2*>(sh);  // [8 warps][8 rows]
+    if (lane < 8) w[8 * warp + lane] = s;
+    __syncthreads();
+    if (threadIdx.x < G) {
+        double2 t = w[threadIdx.x];
+#pragma unroll
+        for (int q = 1; q < kT / 32; ++q) {
+            t.x += w[8 * q + threadIdx.x].x;
+            t.y += w[8 * q + threadIdx.x].y;
+        }
+        fin[threadIdx.x] = t;
+    }
 }
 
 // partial[r][slot][i] over the elements this CTA sweeps, for its group of at
@@ -239,7 +275,6 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
     extern __shared__ __align__(16) unsigned char dsm[];
     TW* ring = reinterpret_cast<TW*>(dsm);  // [kDotStages][kDotG + 1][kT]
     __shared__ double2 red[kDotG][kT / 32];
-    __shared__ double redn[kT / 32];
     const int r = blockIdx.y;
     if (jtab && jtab[r] < 0) return;
     const int nv = rhs_nv(jtab, r, nv_off);
@@ -302,25 +337,36 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
                 sq = E::to_d2(E::warp_reduce(acc[q]));
             if (lane == 0) red[q][warp] = sq;
         }
-    const double wn = (grp == 0) ? warp_sum(E::nfin(wacc)) : 0.0;
-    if (lane == 0) redn[warp] = wn;
-    __syncthreads();
     const int NP = nvmax + 1;
     double2* out = partial + ((long long)r * nslots + slot) * NP;
+    double* sh = reinterpret_cast<double*>(dsm);  // the ring is done with
+    __syncthreads();                              // in every warp, and red is complete
     if (t < G) {
         double2 sum = make_double2(0.0, 0.0);
         for (int q = 0; q < kT / 32; ++q) sum.x += red[t][q].x, sum.y += red[t][q].y;
         out[i0 + t] = sum;
     }
     if (grp == 0) {
-        if (t == 0) {
-            double sum = 0.0;
-            for (int q = 0; q < kT / 32; ++q) sum += redn[q];
-            out[nvmax] = make_double2(sum, 0.0);
-        }
-        for (int i = nv + t; i < nvmax; i += kT) out[i] = make_double2(0.0, 0.0);  // the groups cover [0, nv)
+        const double sum = cta_sum(E::nfin(wacc), sh);
+        if (t == 0) out[nvmax] = make_double2(sum, 0.0);
+        if (!cnt)
+            for (int i = nv + t; i < nvmax; i += kT) out[i] = make_double2(0.0, 0.0);  // the groups cover [0, nv)
     }
-    if (cnt) last_cta_sum(partial + (long long)r * nslots * NP, nslots, NP, cnt + r, fin + (long long)r * NP);
+    if (!cnt) return;
+    // the last CTA of each group reduces the group's rows: the groups' sums run
+    // side by side, and nobody adds rows that this launch has not got
+    if (!last_cta(cnt + r * kMaxGroups + grp, (unsigned)nslots)) return;
+    const double2* part = partial + (long long)r * nslots * NP;
+    double2* fr = fin + (long long)r * NP;
+    group_sum(part + i0, nslots, NP, G, fr + i0, sh);
+    if (grp == 0) {
+        __syncthreads();
+        double s = 0.0;
+        for (int b = t; b < nslots; b += kT) s += __ldcg(&part[(long long)b * NP + nvmax].x);
+        s = cta_sum(s, sh);
+        if (t == 0) fr[nvmax] = make_double2(s, 0.0);
+        for (int i = nv + t; i < nvmax; i += kT) fr[i] = make_double2(0.0, 0.0);
+    }
 }
 
 // out[r][i] = sum_blk partial[r][blk][i]: warp i sums its row lane-strided,

@@ -243,11 +243,14 @@ struct VecRef {
 // out[r][i] = <V_i, w>  (i < nv[r]),  out[r][nvmax] = ||w||^2 ; nv = jtab[r] + nv_off (or nv_off)
 // nv_active: the largest number of basis vectors any rhs has in this launch
 // (sizes the grid); nvmax: the row length of partial/out minus one
-// cnt: nrhs zeroed counters (left zeroed): the last CTA of each rhs sums the
-// partial rows itself; nullptr: a separate reduction launch
+// cnt: zeroed counters (left zeroed), kDotCounters per rhs: the last CTA of each
+// group of vectors sums the group's partial rows itself; nullptr: a separate
+// reduction launch
+constexpr int kDotCounters = 8;
 int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nvmax, int nv_active,
                     int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt = nullptr);
-// w -= sum_i coef[r][i] V_i (i < nv[r]);  out_norm2[r] = ||w||^2 after the update
+// w -= sum_i coef[r][i] V_i (i < nv[r]);  out_norm2[r] = ||w||^2 after the update;
+// cnt as above, one counter per rhs
 int launch_multiaxpy(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nrhs,
                      const double2* coef, int coef_ld, double2* partial, int nblk, double* out_norm2,
                      cudaStream_t st, unsigned* cnt = nullptr);

@@ -73,7 +73,7 @@ struct Solver {
     // device buffers (owned by the workspace of the context)
     char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap, *canon;
     double2 *partial, *dots, *Qd, *etad;
-    unsigned* cnt_d;  // reduction counters of the multi-dot and multi-axpy launches
+    unsigned *cnt_d, *dcnt_d;  // reduction counters of the multi-axpy and multi-dot launches
     double *norm2d, *scal_d;
     int *jtab_d, *nz_d;
     // pinned host mirrors
@@ -228,8 +228,9 @@ int Solver::setup() {
     if ((rc = W->partial.ensure((size_t)nrhs * nblk * NP * sizeof(double2)))) return rc;
     // per-rhs counters of the multi-dot and multi-axpy launches (their last CTA
     // reduces the partial sums and leaves the counter at zero); zeroed per solve
-    if ((rc = W->cnt.ensure((size_t)nrhs * sizeof(unsigned)))) return rc;
-    DW_CUDA_TRY(cudaMemsetAsync(W->cnt.p, 0, (size_t)nrhs * sizeof(unsigned), st));
+    const size_t ncnt = (size_t)nrhs * (1 + kDotCounters);
+    if ((rc = W->cnt.ensure(ncnt * sizeof(unsigned)))) return rc;
+    DW_CUDA_TRY(cudaMemsetAsync(W->cnt.p, 0, ncnt * sizeof(unsigned), st));
     if ((rc = W->dots.ensure((size_t)2 * nrhs * NP * sizeof(double2)))) return rc;
     if ((rc = W->Q.ensure((size_t)(m + 1) * (m + 1) * sizeof(double2)))) return rc;
     if ((rc = W->eta.ensure((size_t)(m + 1) * sizeof(double2)))) return rc;
@@ -267,6 +268,7 @@ int Solver::setup() {
     rlow = (vp != op) ? W->rlow.as<char>() : nullptr;
     partial = W->partial.as<double2>();
     cnt_d = W->cnt.as<unsigned>();
+    dcnt_d = cnt_d + nrhs;
     dots = W->dots.as<double2>();
     Qd = W->Q.as<double2>();
     etad = W->eta.as<double2>();
@@ -341,7 +343,7 @@ int Solver::start_deflated(int r) {
     {
         ProfScope ps(&ctx->prof, "multidot", (double)(mm + 2) * fv);
         if ((rc = launch_multidot(vp, vref_all(r, 0), res_vec(r), n, nullptr, mm + 1, m + 1, mm + 1, 1, partial,
-                                  nblk, dots, st, cnt_d)))
+                                  nblk, dots, st, dcnt_d)))
             return rc;
     }
     DW_CUDA_TRY(cudaMemcpyAsync(dots_h, dots, sizeof(double2) * NP, cudaMemcpyDeviceToHost, st));
@@ -393,7 +395,7 @@ int Solver::start_deflated(int r) {
         ProfScope ps(&ctx->prof, "cgs", (double)(2 * k + 3) * fv);
         VecRef w = vref_all(r, k);
         if ((rc = launch_multidot(vp, vref_all(r, 0), w, n, nullptr, k, m + 1, k, 1, partial, nblk, dots, st,
-                                  cnt_d)))
+                                  dcnt_d)))
             return rc;
         if ((rc = launch_multiaxpy(vp, vref_all(r, 0), w, n, nullptr, k, 1, dots, NP, partial, nblk, norm2d + r,
                                    st, cnt_d)))
@@ -409,7 +411,7 @@ int Solver::start_deflated(int r) {
     {
         ProfScope ps(&ctx->prof, "multidot", (double)(k1 + 1) * fv);
         if ((rc = launch_multidot(vp, vref_all(r, 0), res_vec(r), n, nullptr, k1, m + 1, k1, 1, partial, nblk, dots,
-                                  st, cnt_d)))
+                                  st, dcnt_d)))
             return rc;
     }
     DW_CUDA_TRY(cudaMemcpyAsync(dots_h, dots, sizeof(double2) * NP, cudaMemcpyDeviceToHost, st));
@@ -532,7 +534,7 @@ int Solver::step() {
     {
         ProfScope ps(&ctx->prof, "cgs_project", (jsum + nact) * fv);
         if ((rc = launch_multidot(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, m + 1, jmax + 1, nrhs, partial,
-                                  nblk, dots, st, cnt_d)))
+                                  nblk, dots, st, dcnt_d)))
             return rc;
     }
     {
@@ -570,7 +572,7 @@ int Solver::step() {
         {
             ProfScope ps(&ctx->prof, "cgs_reorth", (2.0 * js2 + 3.0 * n2) * fv);
             if ((rc = launch_multidot(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, m + 1, jmax2 + 1, nrhs,
-                                      partial, nblk, dots, st, cnt_d)))
+                                      partial, nblk, dots, st, dcnt_d)))
                 return rc;
             if ((rc = launch_multiaxpy(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, nrhs, dots, NP, partial,
                                        nblk, norm2d, st, cnt_d)))
