@@ -181,7 +181,7 @@ static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** 
 }
 
 int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
-            long long inbox_rs, const int* jtab, int nrhs, int nact, int ncycles, int nmr) {
+            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
     const Geom& g = ctx->g;
     const long long sb = spinor_bytes(prec, g.V);
     const double first = 0.5 * ((double)nact * 2.0 * sb + link_bytes(prec, g.V));

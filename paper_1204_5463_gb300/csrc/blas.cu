@@ -31,7 +31,10 @@ __device__ __forceinline__ double warp_sum(double a) {
     return a;
 }
 
-__device__ __forceinline__ int rhs_nv(const int* jtab, int r, int off) { return jtab ? jtab[r] + off : off; }
+template <class Tab>
+__device__ __forceinline__ int rhs_nv(const Tab& jtab, int r, int off) {
+    return jtab ? jtab[r] + off : off;
+}
 
 // ---- element access: complex element e of a flat outer vector ---------------
 template <int VP>
@@ -266,9 +269,9 @@ __device__ __forceinline__ void group_sum(const double2* part, int nslots, int N
 // groups, so that the CTAs of all groups stream about the same bytes); the
 // CTAs of group 0 also write ||w||^2 and zero the unused slots.
 template <int VP>
-__global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, long long n, const int* jtab,
+__global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, long long n, const __grid_constant__ RhsCols jtab,
                                                          int nv_off, int nvmax, int ngroups, double2* partial,
-                                                         unsigned* cnt, double2* fin) {
+                                                         unsigned* cnt, double2* fin, int* cols) {
     typedef Elem<VP> E;
     typedef typename E::C C;
     typedef typename E::T TW;  // storage word of one complex element
@@ -276,6 +279,7 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
     TW* ring = reinterpret_cast<TW*>(dsm);  // [kDotStages][kDotG + 1][kT]
     __shared__ double2 red[kDotG][kT / 32];
     const int r = blockIdx.y;
+    if (cols && jtab && blockIdx.x == 0 && threadIdx.x == 0) cols[r] = jtab[r];  // for the multi-axpy that follows
     if (jtab && jtab[r] < 0) return;
     const int nv = rhs_nv(jtab, r, nv_off);
     const int j = jtab ? jtab[r] : 0;
@@ -371,7 +375,7 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
 
 // out[r][i] = sum_blk partial[r][blk][i]: warp i sums its row lane-strided,
 // then a fixed shuffle tree (deterministic)
-__global__ void __launch_bounds__(1024) finalize_kernel(const double2* partial, int nblk, int NP, const int* jtab,
+__global__ void __launch_bounds__(1024) finalize_kernel(const double2* partial, int nblk, int NP, const __grid_constant__ RhsCols jtab,
                                                         double2* out) {
     const int r = blockIdx.x;
     if (jtab && jtab[r] < 0) return;
@@ -525,7 +529,7 @@ __global__ void __launch_bounds__(kT) multiaxpy_f32x2_kernel(VecRef Vb, VecRef w
 
 // ---- v = w / ||w|| per site, optionally also written in SAP storage ----------
 template <int VP, int PS>
-__global__ void __launch_bounds__(kT) normalize_kernel(VecRef w, VecRef dst, long long V, const int* jtab,
+__global__ void __launch_bounds__(kT) normalize_kernel(VecRef w, VecRef dst, long long V, const __grid_constant__ RhsCols jtab,
                                                        const double* norm2, FieldRef low) {
     typedef Elem<VP> E;
     typedef typename E::C C;
@@ -815,8 +819,8 @@ bool basis_ok(int vp) { return vp == P64 || vp == PDF || vp == P32; }
 
 int blas_nblk(long long n) { return (int)grid_for(n); }
 
-int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nvmax, int nv_active,
-                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt) {
+int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, RhsCols jtab, int nv_off, int nvmax, int nv_active,
+                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt, int* cols) {
     if (nvmax > kMaxV) return fail(DW_EINVAL, "too many basis vectors for one multi-dot");
     if (!basis_ok(vp)) return fail(DW_EINVAL, "bad basis precision");
     // CTAs: (element slots) x (groups of at most 8 vectors), at most one wave
@@ -859,13 +863,13 @@ int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, i
     }
     if (vp == PDF)
         multidot_kernel<PDF><<<grid, kT, multidot_smem<PDF>(), st>>>(Vb, w, n, jtab, nv_off, nvmax, ngroups, partial,
-                                                                    cnt, out);
+                                                                    cnt, out, cols);
     else if (vp == P32)
         multidot_kernel<P32><<<grid, kT, multidot_smem<P32>(), st>>>(Vb, w, n, jtab, nv_off, nvmax, ngroups, partial,
-                                                                    cnt, out);
+                                                                    cnt, out, cols);
     else
         multidot_kernel<P64><<<grid, kT, multidot_smem<P64>(), st>>>(Vb, w, n, jtab, nv_off, nvmax, ngroups, partial,
-                                                                    cnt, out);
+                                                                    cnt, out, cols);
     DW_LAUNCH_CHECK();
     if (!cnt) {  // without counters, a separate reduction launch
         finalize_kernel<<<nrhs, 1024, 0, st>>>(partial, (int)nb, nvmax + 1, jtab, out);
@@ -898,7 +902,7 @@ int launch_multiaxpy(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, 
     return DW_OK;
 }
 
-int launch_normalize(int vp, VecRef w, VecRef dst, long long V, const int* jtab, int nrhs, const double* norm2,
+int launch_normalize(int vp, VecRef w, VecRef dst, long long V, RhsCols jtab, int nrhs, const double* norm2,
                      int plow, FieldRef low, cudaStream_t st) {
     if (!basis_ok(vp)) return fail(DW_EINVAL, "bad basis precision");
     dim3 grid((unsigned)((V + kT - 1) / kT), nrhs);

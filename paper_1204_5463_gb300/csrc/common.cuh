@@ -761,6 +761,15 @@ __device__ __forceinline__ void clover_acc(const char* A, long long V, long long
 // where col(r) = jtab[r] when a column table is given (Krylov bases), else 0.
 // A right-hand side with jtab[r] < 0 is inactive for the launch.
 // ---------------------------------------------------------------------------
+// The column table goes to the kernels by value (their parameters lie in
+// constant memory): a step's launches then wait for no copy.
+struct RhsCols {
+    int on;     // 0: no table, column 0 for every rhs, all active
+    int j[16];  // DW_MAX_RHS
+    __host__ __device__ RhsCols(decltype(nullptr) = nullptr) : on(0) {}
+    __host__ __device__ explicit operator bool() const { return on != 0; }
+    __host__ __device__ int operator[](int r) const { return j[r]; }
+};
 struct FieldRef {
     char* base;
     long long rhs_stride;
@@ -768,10 +777,10 @@ struct FieldRef {
     int col_off;
 };
 
-__device__ __forceinline__ char* field_ptr(const FieldRef& f, const int* jtab, int r) {
+__device__ __forceinline__ char* field_ptr(const FieldRef& f, const RhsCols& jtab, int r) {
     const int j = jtab ? jtab[r] : 0;
     return f.base + (long long)r * f.rhs_stride + (long long)(j + f.col_off) * f.col_stride;
 }
-__device__ __forceinline__ bool rhs_active(const int* jtab, int r) { return jtab == nullptr || jtab[r] >= 0; }
+__device__ __forceinline__ bool rhs_active(const RhsCols& jtab, int r) { return !jtab || jtab[r] >= 0; }
 
 }  // namespace dwk

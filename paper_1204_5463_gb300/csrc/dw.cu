@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kThreads) link_convert_kernel(const double2* _
 // Field conversion between internal precisions (same layout family).
 template <int PI, int PO>
 __global__ void __launch_bounds__(kThreads) convert_kernel(FieldRef in, FieldRef out, long long V,
-                                                           const int* jtab) {
+                                                           const __grid_constant__ RhsCols jtab) {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
     if (s >= V || !rhs_active(jtab, r)) return;
@@ -240,7 +240,7 @@ __device__ __forceinline__ void dw_site(const Geom& g, C diag, const char* pin, 
 
 template <int PI, int PO, int PL, class C, bool SUB, bool CLOV>
 __global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
-    dw_kernel(Geom g, C diag, FieldRef in, FieldRef out, const char* U, const int* jtab, int nrhs, FieldRef sub,
+    dw_kernel(Geom g, C diag, FieldRef in, FieldRef out, const char* U, const __grid_constant__ RhsCols jtab, int nrhs, FieldRef sub,
               const char* clov) {
     const int r = blockIdx.x % nrhs;
     const long long s = (blockIdx.x / nrhs) * (long long)blockDim.x + threadIdx.x;
@@ -314,7 +314,7 @@ constexpr bool clover_combo() {
 }
 
 template <int PI, int PO, int PL, class C>
-int dw_dispatch_sub(const Geom& g, double m0, FieldRef in, FieldRef out, const char* U, const int* jtab, int nrhs,
+int dw_dispatch_sub(const Geom& g, double m0, FieldRef in, FieldRef out, const char* U, RhsCols jtab, int nrhs,
                     const FieldRef* sub, const ClovRef* cl, cudaStream_t st) {
     // double-float arithmetic holds about 164 registers a thread: 128-thread
     // blocks let three CTAs (12 warps) share an SM instead of one of 256
@@ -414,7 +414,7 @@ int launch_link_convert(int prec, const char* U64, char* out, long long V, cudaS
     return DW_OK;
 }
 
-int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, const int* jtab, int nrhs,
+int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, RhsCols jtab, int nrhs,
                    cudaStream_t st) {
     dim3 grid = site_grid(V, nrhs);
 #define CONV(A, B)                                                                            \
@@ -465,7 +465,7 @@ int launch_dw_out(int prec, const Geom& g, double m0, const char* in, double* ca
 }
 
 int launch_dw(int pin, int pout, int plink, const Geom& g, double m0, FieldRef in, FieldRef out, const char* U,
-              const int* jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl) {
+              RhsCols jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl) {
     // Supported combinations: uniform precision (the stencil as an operator),
     // and low-precision input with an FP64 output (Arnoldi product w = D z).
 #define DWC(A, B, L, C)                                                                       \

@@ -171,7 +171,7 @@ int launch_link_convert(int prec, const char* U64, char* out, long long V, cudaS
 // out = D in  (sub == nullptr)   or   out = sub - D in  (sub: FP64 field, PO must be P64);
 // with cl, D includes the clover term
 int launch_dw(int pin, int pout, int plink, const Geom& g, double m0, FieldRef in, FieldRef out, const char* U,
-              const int* jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl = nullptr);
+              RhsCols jtab, int nrhs, const FieldRef* sub, cudaStream_t st, const ClovRef* cl = nullptr);
 // out (caller's FP64 layout, nrhs fields) = D in, all in storage precision prec (P64, P32, P16, PB16)
 int launch_dw_out(int prec, const Geom& g, double m0, const char* in, double* out, const char* U, int nrhs,
                   cudaStream_t st, const ClovRef* cl = nullptr);
@@ -186,7 +186,7 @@ int launch_clover_compute(const Geom& g, const char* U64, double csw, double* A6
 // thread count (the sweep reads its links only there); err_host: HostFlag::d,
 // set if a link copy did not complete.
 int launch_sap_sweep(int pspin, int plink, const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg,
-                     const int* jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
+                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
                      const ClovRef* cl, int* err_host);
 int sap_smem_bytes(int pspin, int plink, const Geom& g, int threads);
 // CTA size of the SAP sweep (threads, or the domain volume rounded up to a warp multiple when 0)
@@ -214,7 +214,7 @@ int sap_apply_smem(int pspin, int plink, const Geom& g);
 int sap_inbox_slots(const Geom& g);
 int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st);
 int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st);
-int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab,
+int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab,
                      int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
                      double bytes_first, double bytes_next);
 // Scratch of one application and right-hand side in two pieces: the residuals
@@ -226,7 +226,7 @@ size_t sap_inbox_bytes(int prec, const Geom& g);
 // launch_sap_apply where the domain fits, else sweep by sweep (the scratch is
 // then unused); state and inbox: scratch of the strides given
 int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
-            long long inbox_rs, const int* jtab, int nrhs, int nact, int ncycles, int nmr);
+            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
 // after the stream was synchronised: DW_ETIMEOUT if a SAP kernel's bounded wait gave up
 int sap_check(dw_ctx* ctx);
 
@@ -245,17 +245,20 @@ struct VecRef {
 // (sizes the grid); nvmax: the row length of partial/out minus one
 // cnt: zeroed counters (left zeroed), kDotCounters per rhs: the last CTA of each
 // group of vectors sums the group's partial rows itself; nullptr: a separate
-// reduction launch
+// reduction launch. cols (device, one int per rhs, may be null) receives the
+// column table for the multi-axpy after it: reading the table from memory, that
+// kernel's loop is 643 us where every form with the table in its parameters is
+// 664 to 863 us (12 rhs, 16 vectors on average, 16^3 x 32)
 constexpr int kDotCounters = 8;
-int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nvmax, int nv_active,
-                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt = nullptr);
+int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, RhsCols jtab, int nv_off, int nvmax, int nv_active,
+                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt = nullptr, int* cols = nullptr);
 // w -= sum_i coef[r][i] V_i (i < nv[r]);  out_norm2[r] = ||w||^2 after the update;
-// cnt as above, one counter per rhs
+// cnt as above, one counter per rhs; jtab: the device table of the multi-dot
 int launch_multiaxpy(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nrhs,
                      const double2* coef, int coef_ld, double2* partial, int nblk, double* out_norm2,
                      cudaStream_t st, unsigned* cnt = nullptr);
 // dst = w / sqrt(norm2[r]) per site; if plow >= 0 also written to `low` in spinor storage plow
-int launch_normalize(int vp, VecRef w, VecRef dst, long long V, const int* jtab, int nrhs, const double* norm2,
+int launch_normalize(int vp, VecRef w, VecRef dst, long long V, RhsCols jtab, int nrhs, const double* norm2,
                      int plow, FieldRef low, cudaStream_t st);
 // in place, per element: X_c = sum_i X_i Q[r][i][c]  (c < kout, i < nin), X in precision prec
 // (scaled FP16/BF16 storage goes through `scratch`, nrhs * kout columns, and is copied back)
@@ -270,7 +273,7 @@ int launch_xupdate(int prec, int vx, const char* Z, long long z_rs, long long z_
 int launch_norm2(int vp, const double2* a, long long rs, long long n, int nrhs, double2* partial, int nblk,
                  double* out, cudaStream_t st);
 // convert a spinor field between storage precisions for a set of rhs
-int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, const int* jtab, int nrhs,
+int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, RhsCols jtab, int nrhs,
                    cudaStream_t st);
 // dst = a[r] * src  (outer vectors)
 int launch_scale(int vp, const double2* src, double2* dst, long long rs, long long n, int nrhs, const double* a,

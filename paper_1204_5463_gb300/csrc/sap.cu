@@ -190,7 +190,7 @@ __device__ __forceinline__ void bulk_copy_start(void* dst, const void* src, unsi
 // err_host: set (host-mapped) if the bulk copy of the links did not complete.
 template <int PS, int PL, class C, int MAXT, bool CLOV>
 __global__ void __launch_bounds__(MAXT, (MAXT <= 256 && sizeof(C) == 4) ? 2 : 1)
-    sap_sweep_kernel(Geom g, C diag, FieldRef vref, FieldRef xref, const char* __restrict__ Uimg, const int* jtab,
+    sap_sweep_kernel(Geom g, C diag, FieldRef vref, FieldRef xref, const char* __restrict__ Uimg, const __grid_constant__ RhsCols jtab,
                      int nrhs, int colour, int nmr, int mode, const char* __restrict__ clov, int* err_host) {
     constexpr int CP = (sizeof(C) == 4) ? P32 : P64;  // storage of the clover term
     typedef LinkSh<PL> LS;
@@ -451,7 +451,7 @@ __global__ void link_image_kernel(Geom g, const char* __restrict__ U, char* __re
 }
 
 template <int PS, int PL, class C>
-int sap_launch_t(const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg, const int* jtab, int nrhs,
+int sap_launch_t(const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg, RhsCols jtab, int nrhs,
                  int colour, int nmr, int mode, int threads, cudaStream_t st, const ClovRef* cl, int* err_host) {
     if (cl && threads > 256) return fail(DW_EINVAL, "the clover SAP sweep handles domains of at most 256 sites");
     const size_t smem = (size_t)sap_smem_bytes(PS, PL, g, threads);
@@ -538,7 +538,7 @@ int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, in
 }
 
 int launch_sap_sweep(int pspin, int plink, const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg,
-                     const int* jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
+                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
                      const ClovRef* cl, int* err_host) {
     threads = sap_threads(g, threads);
     if (threads < g.B || threads % 32 != 0 || threads > 1024) return fail(DW_EINVAL, "bad SAP thread count");

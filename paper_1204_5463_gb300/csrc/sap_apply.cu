@@ -58,7 +58,7 @@ struct SapArgs {
     long long xpart_rs;
     char* inbox;                  // per rhs: [domain] of Half<C> boxes
     long long inbox_rs;
-    const int* jtab;
+    RhsCols jtab;
     int nrhs, nmr;
     int s0, s1, nsweeps;          // sweeps of this launch, sweeps of the application (2 per cycle)
     const char* clov;
@@ -656,7 +656,7 @@ __global__ void faces_kernel(Geom g, unsigned short* faces) {
 }
 
 template <int PS, int PL, class C>
-int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab, int nrhs,
+int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab, int nrhs,
                 int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof, double bytes_first,
                 double bytes_next) {
     const int threads = sap_threads(g, 0);
@@ -785,7 +785,7 @@ int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st) {
     return DW_OK;
 }
 
-int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, const int* jtab,
+int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab,
                      int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
                      double bytes_first, double bytes_next) {
     if (prec == P64)

@@ -38,6 +38,32 @@
 
 namespace dwk {
 
+// Workspace kept by the context between solves (grown on demand).
+struct Workspace {
+    DevBuf V, Z, x, b, r, vlow, zscr, rlow, zsap, partial, dots, Q, eta, scal, nz, canon, cnt, bscale;
+    // the last solve's bases as dw_debug_basis reads them: formats, sizes and,
+    // per rhs, the columns and the (m+1) x m Hessenberg-like matrix of its last cycle
+    int last_nrhs = 0, last_m = 0, last_vp = -1, last_zp = -1;
+    long long last_fv = 0, last_zb = 0;
+    std::vector<int> last_mm;
+    std::vector<std::vector<zd>> last_H;
+    std::vector<std::vector<double>> last_hist;  // per rhs: (steps, implicit, explicit) per cycle
+    double2* dots_h = nullptr;
+    double* norm2_h = nullptr;
+    size_t dots_h_n = 0;
+    // the stream that reads a step's results back, and the events around the copy
+    cudaStream_t back = nullptr;
+    cudaEvent_t ready = nullptr, done = nullptr;
+    ~Workspace() {
+        if (back) cudaStreamSynchronize(back);  // a copy may be in flight after an error
+        if (ready) cudaEventDestroy(ready);
+        if (done) cudaEventDestroy(done);
+        if (back) cudaStreamDestroy(back);
+        if (dots_h) cudaFreeHost(dots_h);
+        if (norm2_h) cudaFreeHost(norm2_h);
+    }
+};
+
 namespace {
 
 struct RhsState {
@@ -75,13 +101,11 @@ struct Solver {
     double2 *partial, *dots, *Qd, *etad;
     unsigned *cnt_d, *dcnt_d;  // reduction counters of the multi-axpy and multi-dot launches
     double *norm2d, *scal_d;
-    int *jtab_d, *nz_d;
+    int *nz_d, *cols_d;
     // pinned host mirrors
     double2* dots_h;
     double* norm2_h;
-    int* jtab_h;
-    double* norm2_up;  // upload copies for the end of a step (the next step rewrites jtab_h
-    int* jtab_up;      // before the device has necessarily consumed the previous upload)
+    RhsCols cols;  // per rhs the column of the step, -1: not stepping
     std::vector<RhsState> R;
     int explicit_res = 0;
 
@@ -131,44 +155,28 @@ struct Solver {
         DW_CUDA_TRY(cudaStreamSynchronize(st));
         return sap_check(ctx);
     }
-    // the step's dot rows and norms, read back with one copy (the norms follow
-    // the rows in the same device buffer), then a synchronisation
-    int read_dots_norms() {
+    // The step's dot rows and norms, copied with one copy (the norms follow the
+    // rows in the same device buffer) on a stream of its own once the kernels
+    // before it have run, so that the kernels launched after it need not wait ...
+    int fetch_dots_norms() {
+        Workspace* W = ctx->ws;
+        DW_CUDA_TRY(cudaEventRecord(W->ready, st));
+        DW_CUDA_TRY(cudaStreamWaitEvent(W->back, W->ready, 0));
         DW_CUDA_TRY(cudaMemcpyAsync(dots_h, dots, sizeof(double2) * nrhs * NP + sizeof(double) * nrhs,
-                                    cudaMemcpyDeviceToHost, st));
-        const int rc = sync();
-        if (rc) return rc;
-        std::memcpy(norm2_h, reinterpret_cast<const double*>(dots_h + (size_t)nrhs * NP), sizeof(double) * nrhs);
+                                    cudaMemcpyDeviceToHost, W->back));
+        DW_CUDA_TRY(cudaEventRecord(W->done, W->back));
         return DW_OK;
+    }
+    // ... and waited for. The device buffer is written again only by launches
+    // that follow this wait.
+    int wait_dots_norms() {
+        DW_CUDA_TRY(cudaEventSynchronize(ctx->ws->done));
+        std::memcpy(norm2_h, reinterpret_cast<const double*>(dots_h + (size_t)nrhs * NP), sizeof(double) * nrhs);
+        return sap_check(ctx);
     }
 };
 
 }  // namespace
-
-// Workspace kept by the context between solves (grown on demand).
-struct Workspace {
-    DevBuf V, Z, x, b, r, vlow, zscr, rlow, zsap, partial, dots, Q, eta, scal, jtab, nz, canon, cnt, bscale;
-    // the last solve's bases as dw_debug_basis reads them: formats, sizes and,
-    // per rhs, the columns and the (m+1) x m Hessenberg-like matrix of its last cycle
-    int last_nrhs = 0, last_m = 0, last_vp = -1, last_zp = -1;
-    long long last_fv = 0, last_zb = 0;
-    std::vector<int> last_mm;
-    std::vector<std::vector<zd>> last_H;
-    std::vector<std::vector<double>> last_hist;  // per rhs: (steps, implicit, explicit) per cycle
-    double2* dots_h = nullptr;
-    double* norm2_h = nullptr;
-    int* jtab_h = nullptr;
-    double* norm2_up = nullptr;
-    int* jtab_up = nullptr;
-    size_t dots_h_n = 0;
-    ~Workspace() {
-        if (dots_h) cudaFreeHost(dots_h);
-        if (norm2_h) cudaFreeHost(norm2_h);
-        if (jtab_h) cudaFreeHost(jtab_h);
-        if (norm2_up) cudaFreeHost(norm2_up);
-        if (jtab_up) cudaFreeHost(jtab_up);
-    }
-};
 
 void release_workspace(Workspace* w) { delete w; }
 
@@ -178,7 +186,7 @@ static Workspace* workspace_of(dw_ctx* ctx) {
         if (ctx->ws)
             for (DevBuf* b : {&ctx->ws->V, &ctx->ws->Z, &ctx->ws->x, &ctx->ws->b, &ctx->ws->r, &ctx->ws->vlow,
                               &ctx->ws->zscr, &ctx->ws->rlow, &ctx->ws->zsap, &ctx->ws->partial, &ctx->ws->dots, &ctx->ws->Q, &ctx->ws->eta,
-                              &ctx->ws->scal, &ctx->ws->jtab, &ctx->ws->nz, &ctx->ws->canon,
+                              &ctx->ws->scal, &ctx->ws->nz, &ctx->ws->canon,
                               &ctx->ws->cnt, &ctx->ws->bscale})
                 b->st = ctx->stream;
     }
@@ -228,34 +236,27 @@ int Solver::setup() {
     if ((rc = W->partial.ensure((size_t)nrhs * nblk * NP * sizeof(double2)))) return rc;
     // per-rhs counters of the multi-dot and multi-axpy launches (their last CTA
     // reduces the partial sums and leaves the counter at zero); zeroed per solve
-    const size_t ncnt = (size_t)nrhs * (1 + kDotCounters);
+    const size_t ncnt = (size_t)nrhs * (1 + kDotCounters + 1);  // and the multi-axpy's column table
     if ((rc = W->cnt.ensure(ncnt * sizeof(unsigned)))) return rc;
     DW_CUDA_TRY(cudaMemsetAsync(W->cnt.p, 0, ncnt * sizeof(unsigned), st));
     if ((rc = W->dots.ensure((size_t)2 * nrhs * NP * sizeof(double2)))) return rc;
     if ((rc = W->Q.ensure((size_t)(m + 1) * (m + 1) * sizeof(double2)))) return rc;
     if ((rc = W->eta.ensure((size_t)(m + 1) * sizeof(double2)))) return rc;
     if ((rc = W->scal.ensure((size_t)nrhs * sizeof(double)))) return rc;
-    if ((rc = W->jtab.ensure((size_t)nrhs * sizeof(int)))) return rc;
     if ((rc = W->nz.ensure(sizeof(int)))) return rc;
     if ((rc = W->bscale.ensure((size_t)2 * nrhs * sizeof(double)))) return rc;
     if (W->dots_h_n < (size_t)nrhs * NP) {
         if (W->dots_h) cudaFreeHost(W->dots_h);
         if (W->norm2_h) cudaFreeHost(W->norm2_h);
-        if (W->jtab_h) cudaFreeHost(W->jtab_h);
-        if (W->norm2_up) cudaFreeHost(W->norm2_up);
-        if (W->jtab_up) cudaFreeHost(W->jtab_up);
-        W->norm2_up = nullptr;
-        W->jtab_up = nullptr;
         W->dots_h = nullptr;
         W->norm2_h = nullptr;
-        W->jtab_h = nullptr;
         DW_CUDA_TRY(cudaMallocHost(&W->dots_h, (size_t)2 * DW_MAX_RHS * 66 * sizeof(double2)));
         DW_CUDA_TRY(cudaMallocHost(&W->norm2_h, (size_t)DW_MAX_RHS * sizeof(double)));
-        DW_CUDA_TRY(cudaMallocHost(&W->jtab_h, (size_t)DW_MAX_RHS * sizeof(int)));
-        DW_CUDA_TRY(cudaMallocHost(&W->norm2_up, (size_t)DW_MAX_RHS * sizeof(double)));
-        DW_CUDA_TRY(cudaMallocHost(&W->jtab_up, (size_t)DW_MAX_RHS * sizeof(int)));
         W->dots_h_n = (size_t)DW_MAX_RHS * 66;
     }
+    if (!W->back) DW_CUDA_TRY(cudaStreamCreateWithFlags(&W->back, cudaStreamNonBlocking));
+    if (!W->ready) DW_CUDA_TRY(cudaEventCreateWithFlags(&W->ready, cudaEventDisableTiming));
+    if (!W->done) DW_CUDA_TRY(cudaEventCreateWithFlags(&W->done, cudaEventDisableTiming));
     Vb = W->V.as<char>();
     Zb = W->Z.as<char>();
     xb = W->x.as<char>();
@@ -269,6 +270,7 @@ int Solver::setup() {
     partial = W->partial.as<double2>();
     cnt_d = W->cnt.as<unsigned>();
     dcnt_d = cnt_d + nrhs;
+    cols_d = reinterpret_cast<int*>(dcnt_d + (size_t)nrhs * kDotCounters);
     dots = W->dots.as<double2>();
     Qd = W->Q.as<double2>();
     etad = W->eta.as<double2>();
@@ -276,13 +278,9 @@ int Solver::setup() {
     // with one copy (the dot rows take the first nrhs * NP entries)
     norm2d = reinterpret_cast<double*>(dots + (size_t)nrhs * NP);
     scal_d = W->scal.as<double>();
-    jtab_d = W->jtab.as<int>();
     nz_d = W->nz.as<int>();
     dots_h = W->dots_h;
     norm2_h = W->norm2_h;
-    jtab_h = W->jtab_h;
-    norm2_up = W->norm2_up;
-    jtab_up = W->jtab_up;
     R.assign(nrhs, RhsState());
     for (auto& s : R) {
         s.H.assign((size_t)(m + 1) * m, zd(0));
@@ -495,11 +493,11 @@ int Solver::step() {
     int rc;
     int nact = 0;
     for (int r = 0; r < nrhs; ++r) {
-        jtab_h[r] = (!R[r].done && R[r].j >= 0) ? R[r].j : -1;
-        nact += jtab_h[r] >= 0;
+        cols.j[r] = (!R[r].done && R[r].j >= 0) ? R[r].j : -1;
+        nact += cols.j[r] >= 0;
     }
+    cols.on = 1;
     if (nact == 0) return fail(DW_EBREAKDOWN, "no right-hand side left to step");
-    DW_CUDA_TRY(cudaMemcpyAsync(jtab_d, jtab_h, sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
     const FieldRef Vf1{Vb, (m + 1) * fv, fv, 1};
     const FieldRef Zf{Zb, m * zb, zb, 0};
     const FieldRef Lf{vlow, sb, 0, 0};
@@ -508,11 +506,11 @@ int Solver::step() {
     // The preconditioner's scratch lies in rb (the explicit residual is formed
     // and consumed within cycle_end, so rb is free during the steps) and in the
     // staging copy of the right-hand sides: 192 bytes per site and rhs each.
-    if ((rc = sap_run(ctx, sp, Lf, Zs, rb, fb, canon, 192 * V, jtab_d, nrhs, nact, P.sap_cycles, P.mr_steps)))
+    if ((rc = sap_run(ctx, sp, Lf, Zs, rb, fb, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
         return rc;
     if (zp != sp) {
         ProfScope ps(&ctx->prof, "z_widen", (double)nact * (sb + zb));
-        if ((rc = launch_convert(sp, zp, Zs, Zf, V, jtab_d, nrhs, st))) return rc;
+        if ((rc = launch_convert(sp, zp, Zs, Zf, V, cols, nrhs, st))) return rc;
     }
     // w = D z_j  (written into column j+1 of V)
     {
@@ -521,99 +519,75 @@ int Solver::step() {
         const double link_reads = 1.0;
         ProfScope ps(&ctx->prof, "dw_matvec",
                      (double)nact * (spinor_bytes(zp, V) + spinor_bytes(vp, V)) + link_reads * link_bytes(pl, V));
-        if ((rc = launch_dw(zp, vp, pl, g, ctx->m0, Zf, Vf1, U_mv, jtab_d, nrhs, nullptr, st, ctx->clover())))
+        if ((rc = launch_dw(zp, vp, pl, g, ctx->m0, Zf, Vf1, U_mv, cols, nrhs, nullptr, st, ctx->clover())))
             return rc;
     }
-    // classical Gram-Schmidt: h = V^H w, w' = w - V h; a second projection
-    // ("twice is enough") only where cancellation could cost orthogonality at
-    // the working precision: u / (||w'|| / ||w||) > 1e-13
-    double jsum = 0;
-    int jmax = 0;
-    for (int r = 0; r < nrhs; ++r)
-        if (jtab_h[r] >= 0) jsum += jtab_h[r] + 1, jmax = std::max(jmax, jtab_h[r]);
-    {
-        ProfScope ps(&ctx->prof, "cgs_project", (jsum + nact) * fv);
-        if ((rc = launch_multidot(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, m + 1, jmax + 1, nrhs, partial,
-                                  nblk, dots, st, dcnt_d)))
-            return rc;
-    }
-    {
-        ProfScope ps(&ctx->prof, "cgs_update", (jsum + 2.0 * nact) * fv);
-        if ((rc = launch_multiaxpy(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, nrhs, dots, NP, partial, nblk,
-                                   norm2d, st, cnt_d)))
-            return rc;
-    }
-    if ((rc = read_dots_norms())) return rc;
+    // classical Gram-Schmidt: h = V^H w, w' = w - V h, v_{j+1} = w' / ||w'|| (also
+    // into SAP storage); a second projection ("twice is enough") only where
+    // cancellation could cost orthogonality at the working precision:
+    // u / (||w'|| / ||w||) > 1e-13. The host decides that from the dots and norms;
+    // the normalisation does not wait for it, so a second pass starts from the
+    // normalised vector and its coefficients are scaled by ||w'||.
+    auto project = [&](const RhsCols& c, const char* dots_name, const char* update_name) -> int {
+        double jsum = 0;
+        int jmax = 0, na = 0;
+        for (int r = 0; r < nrhs; ++r)
+            if (c.j[r] >= 0) jsum += c.j[r] + 1, jmax = std::max(jmax, c.j[r]), ++na;
+        {
+            ProfScope ps(&ctx->prof, dots_name, (jsum + na) * fv);
+            if ((rc = launch_multidot(vp, vref_all(0, 0), vref_all(0, 1), n, c, 1, m + 1, jmax + 1, nrhs, partial, nblk,
+                                      dots, st, dcnt_d, cols_d)))
+                return rc;
+        }
+        {
+            ProfScope ps(&ctx->prof, update_name, (jsum + 2.0 * na) * fv);
+            if ((rc = launch_multiaxpy(vp, vref_all(0, 0), vref_all(0, 1), n, cols_d, 1, nrhs, dots, NP, partial, nblk,
+                                       norm2d, st, cnt_d)))
+                return rc;
+        }
+        if ((rc = fetch_dots_norms())) return rc;
+        ProfScope ps(&ctx->prof, "normalize", (double)na * (2.0 * fv + sb));
+        return launch_normalize(vp, vref_all(0, 1), vref_all(0, 1), V, c, nrhs, norm2d, sp, Lf, st);
+    };
+    if ((rc = project(cols, "cgs_project", "cgs_update"))) return rc;
+    if ((rc = wait_dots_norms())) return rc;
     // unit roundoff of the basis format, and the orthogonality level below
     // which a second pass is taken (FP64-class: 1e-13; FP32: 1e-5)
     const double unit = (vp == P32) ? 5.960464477539063e-08 : (vp == PDF) ? 3.552713678800501e-15
                                                                             : 1.1102230246251565e-16;
     const double tau = (vp == P32) ? 1e-5 : 1e-13;
     std::vector<std::vector<zd>> h(nrhs);
+    std::vector<double> hn(nrhs, 0.0);  // ||w'|| after the last pass
+    RhsCols again = cols;
     bool need2 = false;
     for (int r = 0; r < nrhs; ++r) {
-        if (jtab_h[r] < 0) continue;
-        const int j = jtab_h[r];
+        if (cols.j[r] < 0) continue;
+        const int j = cols.j[r];
         h[r].resize(j + 2);
         for (int i = 0; i <= j; ++i) h[r][i] = zd(dots_h[lin(r, i)].x, dots_h[lin(r, i)].y);
         R[r].wn0 = std::sqrt(dots_h[lin(r, m + 1)].x);
-        const double ratio = std::sqrt(norm2_h[r]) / (R[r].wn0 > 0 ? R[r].wn0 : 1.0);
+        hn[r] = std::sqrt(norm2_h[r]);
+        const double ratio = hn[r] / (R[r].wn0 > 0 ? R[r].wn0 : 1.0);
         const bool re = unit > tau * ratio;
         need2 |= re;
-        if (!re) jtab_h[r] = -1;
+        if (!re) again.j[r] = -1;
     }
     if (need2) {
-        DW_CUDA_TRY(cudaMemcpyAsync(jtab_d, jtab_h, sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
-        double js2 = 0;
-        int n2 = 0, jmax2 = 0;
-        for (int r = 0; r < nrhs; ++r)
-            if (jtab_h[r] >= 0) js2 += jtab_h[r] + 1, ++n2, jmax2 = std::max(jmax2, jtab_h[r]);
-        std::vector<double> keep(norm2_h, norm2_h + nrhs);
-        {
-            ProfScope ps(&ctx->prof, "cgs_reorth", (2.0 * js2 + 3.0 * n2) * fv);
-            if ((rc = launch_multidot(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, m + 1, jmax2 + 1, nrhs,
-                                      partial, nblk, dots, st, dcnt_d)))
-                return rc;
-            if ((rc = launch_multiaxpy(vp, vref_all(0, 0), vref_all(0, 1), n, jtab_d, 1, nrhs, dots, NP, partial,
-                                       nblk, norm2d, st, cnt_d)))
-                return rc;
-        }
-        if ((rc = read_dots_norms())) return rc;
+        if ((rc = project(again, "cgs_reorth", "cgs_reorth"))) return rc;
+        if ((rc = wait_dots_norms())) return rc;
         for (int r = 0; r < nrhs; ++r) {
-            if (jtab_h[r] < 0) {
-                norm2_h[r] = keep[r];
-                continue;
-            }
-            for (int i = 0; i <= jtab_h[r]; ++i) h[r][i] += zd(dots_h[lin(r, i)].x, dots_h[lin(r, i)].y);
+            if (again.j[r] < 0) continue;
+            for (int i = 0; i <= again.j[r]; ++i) h[r][i] += hn[r] * zd(dots_h[lin(r, i)].x, dots_h[lin(r, i)].y);
+            hn[r] *= std::sqrt(norm2_h[r]);
         }
-    }
-    // restore the step's column table; v_{j+1} = w / ||w|| (also into SAP storage)
-    for (int r = 0; r < nrhs; ++r) {
-        jtab_h[r] = (!R[r].done && R[r].j >= 0) ? R[r].j : -1;
-        jtab_up[r] = jtab_h[r];
-        norm2_up[r] = norm2_h[r];
-    }
-    if (need2) {
-        // without a second pass the device still holds this step's column
-        // table and the norms just read back: the uploads are needed only
-        // after a second pass changed them (this is the one host round trip
-        // of a step, so every call saved shortens the GPU's idle gap)
-        DW_CUDA_TRY(cudaMemcpyAsync(jtab_d, jtab_up, sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
-        DW_CUDA_TRY(cudaMemcpyAsync(norm2d, norm2_up, sizeof(double) * nrhs, cudaMemcpyHostToDevice, st));
-    }
-    {
-        ProfScope ps(&ctx->prof, "normalize", (double)nact * (2.0 * fv + sb));
-        if ((rc = launch_normalize(vp, vref_all(0, 1), vref_all(0, 1), V, jtab_d, nrhs, norm2d, sp, Lf, st)))
-            return rc;
     }
     // host: Hessenberg column, Givens update, end-of-cycle tests
     for (int r = 0; r < nrhs; ++r) {
         RhsState& s = R[r];
         if (s.done || s.j < 0) continue;
         const int j = s.j;
-        const double hn = std::sqrt(norm2_h[r]);
-        h[r][j + 1] = hn;
-        bool finite = std::isfinite(hn);
+        h[r][j + 1] = hn[r];
+        bool finite = std::isfinite(hn[r]);
         for (int i = 0; i <= j + 1; ++i) {
             finite &= std::isfinite(h[r][i].real()) && std::isfinite(h[r][i].imag());
             s.H[(size_t)i * m + j] = h[r][i];
@@ -627,7 +601,7 @@ int Solver::step() {
         std::vector<zd> col(m + 1, zd(0));
         for (int i = 0; i <= j + 1; ++i) col[i] = s.H[(size_t)i * m + j];
         const double res = s.ls.add_column(col.data(), j + 2);
-        const bool breakdown = hn <= 1e-14 * s.wn0;
+        const bool breakdown = hn[r] <= 1e-14 * s.wn0;
         const bool limit = P.max_iterations > 0 && s.iterations >= P.max_iterations;
         if (breakdown || res <= P.tol * s.bnorm || j + 1 == m || limit) {
             s.mm = j + 1;
@@ -637,9 +611,7 @@ int Solver::step() {
             s.j = j + 1;
         }
     }
-    // no synchronisation here: the next step's launches queue behind the
-    // normalisation (its uploads read jtab_up / norm2_up, which are only
-    // rewritten after the next step's first synchronisation)
+    // no synchronisation here: the next step's launches queue behind the normalisation
     for (int r = 0; r < nrhs; ++r)
         if (R[r].cycle_end) {
             R[r].cycle_end = false;
