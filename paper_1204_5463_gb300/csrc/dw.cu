@@ -170,12 +170,11 @@ __global__ void __launch_bounds__(kThreads) convert_kernel(FieldRef in, FieldRef
 }
 
 // CTAs per SM (measured at 24^3 x 48): the FP32 stencil is latency-bound and
-// fastest at three (80 registers), the 16-bit one is issue-bound (decode) and
-// fastest at two (no register cap that forces spills), the Arnoldi product
-// (FP32 in, double-float out) at four; other 16-bit inputs keep three
+// fastest at three (80 registers), the Arnoldi product (FP32 in, double-float
+// out) at four; 16-bit inputs run at three
 template <int PI, int PO, int PL, class C>
 constexpr int dw_min_blocks() {
-    return sizeof(C) != 4 ? 1 : (PI == P32 && PO == P32) ? 3 : (PI == P32) ? 4 : (PO == PI) ? 2 : 3;
+    return sizeof(C) != 4 ? 1 : (PI == P32 && PO == P32) ? 3 : (PI == P32) ? 4 : 3;
 }
 
 // D at one site, diag psi - 1/2 hops (the clover term included), or b minus
@@ -258,11 +257,12 @@ __global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
 // writes 64 contiguous bytes of each site and the tile stays small beside L1,
 // on which the stencil lives. Stencil and conversion apart and together, 24^3 x
 // 48: FP32 one field 64 + 32 -> 81 us (HBM and latency), twelve FP16 fields 565
-// + 280 -> 790 us (instructions: 24 conversions and 24 scalings of every
+// + 280 -> 722 us (three CTAs an SM; two 790, and two fields a thread sharing
+// the decoded links 719; instructions: 24 conversions and 24 scalings of every
 // neighbour); FP64 at 16^3 x 32 318 + 10 -> 232 us with hop_pair (the FP64 pipe:
 // 840 instructions a site take 190 us).
 template <int P, class C, bool CLOV>
-__global__ void __launch_bounds__(kThreads, dw_min_blocks<P, P, P, C>())
+__global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 3 : 1)
     dw_out_kernel(Geom g, C diag, const char* in, long long in_rs, double* canon, const char* U, int nrhs,
                   const char* clov) {
     __shared__ __align__(16) double2 tiles[kThreads / 32][32 * 5];
