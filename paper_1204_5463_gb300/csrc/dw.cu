@@ -305,6 +305,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 3 : 1)
     }
 }
 
+// Threads of a stencil block: the largest power of two up to `most` with which
+// the blocks still go round the SMs twice (a lattice of a few thousand sites
+// otherwise keeps a handful of SMs busy: FP64 at 4^4, whose pipe takes 50 us for
+// 256 sites, 72 -> 44 us a call, FP32 19.8 -> 19.1). At least a warp.
+int stencil_threads(long long V, int nrhs, int most) {
+    int t = most;
+    while (t > 32 && (V + t - 1) / t * nrhs < 2 * 152) t >>= 1;
+    return t;
+}
+
 dim3 site_grid(long long V, int nrhs) { return dim3((unsigned)((V + kThreads - 1) / kThreads), nrhs); }
 
 // every supported precision combination carries the clover term
@@ -318,7 +328,7 @@ int dw_dispatch_sub(const Geom& g, double m0, FieldRef in, FieldRef out, const c
                     const FieldRef* sub, const ClovRef* cl, cudaStream_t st) {
     // double-float arithmetic holds about 164 registers a thread: 128-thread
     // blocks let three CTAs (12 warps) share an SM instead of one of 256
-    constexpr int bt = std::is_same<C, df>::value ? 128 : kThreads;
+    const int bt = stencil_threads(g.V, nrhs, std::is_same<C, df>::value ? 128 : kThreads);
     const unsigned nb = (unsigned)((g.V + bt - 1) / bt) * (unsigned)nrhs;
     const C diag = C(4.0 + m0);
     FieldRef none{};
@@ -443,16 +453,17 @@ int launch_convert(int pin, int pout, FieldRef in, FieldRef out, long long V, Rh
 
 int launch_dw_out(int prec, const Geom& g, double m0, const char* in, double* canon, const char* U, int nrhs,
                   cudaStream_t st, const ClovRef* cl) {
-    const unsigned nb = (unsigned)((g.V + kThreads - 1) / kThreads) * (unsigned)nrhs;
+    const int bt = stencil_threads(g.V, nrhs, kThreads);
+    const unsigned nb = (unsigned)((g.V + bt - 1) / bt) * (unsigned)nrhs;
     const long long rs = spinor_bytes(prec, g.V);
     const double d = 4.0 + m0;
 #define DWO(P, C)                                                                                                 \
     if (prec == P) {                                                                                              \
         const char* A = cl ? ((sizeof(C) == 4) ? cl->a32 : cl->a64) : nullptr;                                    \
         if (cl)                                                                                                   \
-            dw_out_kernel<P, C, true><<<nb, kThreads, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);               \
+            dw_out_kernel<P, C, true><<<nb, bt, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);               \
         else                                                                                                      \
-            dw_out_kernel<P, C, false><<<nb, kThreads, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);              \
+            dw_out_kernel<P, C, false><<<nb, bt, 0, st>>>(g, C(d), in, rs, canon, U, nrhs, A);              \
         DW_LAUNCH_CHECK();                                                                                        \
         return DW_OK;                                                                                             \
     }
