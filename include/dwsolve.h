@@ -23,7 +23,9 @@
  * Every call returns DW_OK (0) or a DW_E* code; dw_last_error() gives a
  * message for the calling thread. No C++ exception crosses this boundary.
  * All device work of a context is issued on the CUDA stream given to
- * dw_create; calls return after that work has completed unless stated.
+ * dw_create (a solve reads each Arnoldi step's results back on a stream of its
+ * own, ordered after that work); calls return after that work has completed
+ * unless stated.
  */
 #ifndef DWSOLVE_H
 #define DWSOLVE_H
@@ -113,13 +115,16 @@ int dw_apply(dw_ctx* ctx, const double* in, double* out, dw_prec prec, int nrhs)
 /* z = M v with M the SAP preconditioner (Sec. 4): ncycles iterations of
  * Algorithm 2 started from x = 0, each a sweep over the domains of colour 0
  * (block coordinates summing to an even number; contains site 0) followed by
- * colour 1. Each domain solve computes r = (v - D x)^l with the full
- * operator, runs nmr minimal-residual steps on D^l y = r from y = 0 (Sec. 4)
- * and adds x^l += y^l. storage selects the precision of v, x and the links
+ * colour 1. Each domain solve starts from r = (v - D x)^l of the full
+ * operator (carried from visit to visit with the neighbours' corrections, or
+ * recomputed for domains whose halo does not fit), runs nmr minimal-residual
+ * steps on D^l y = r from y = 0 (Sec. 4) and adds x^l += y^l. storage selects the precision of v, x and the links
  * (arithmetic FP32 for DW_F32/F16/BF16, FP64 for DW_F64).
  * v, z: device pointers, canonical FP64 layout, nrhs fields each.
  * Requires ncycles >= 1, nmr >= 1. Each domain's CTA waits (at most about a
- * second) for the bulk copy of its links; if a wait gives up the call, and a
+ * second) for the bulk copy of its links, and where all domains run as one
+ * cooperative launch (at most about two seconds and 0.2 ms per MR step) for
+ * the previous sweep; if a wait gives up the call, and a
  * solve whose preconditioner it was, returns DW_ETIMEOUT.
  * Errors: DW_EINVAL, DW_ENOMEM, DW_ECUDA, DW_ETIMEOUT. */
 int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int nmr, dw_prec storage, int nrhs);

@@ -32,6 +32,7 @@
 // latency of shared memory at the 16 warps that 128 registers allow, with its
 // pipe busy three quarters of the time; paired, scalar and mixed forms of the
 // hop's FP32 arithmetic are within 2% of one another.
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -62,6 +63,7 @@ struct SapArgs {
     int nrhs, nmr;
     int s0, s1, nsweeps;          // sweeps of this launch, sweeps of the application (2 per cycle)
     const char* clov;
+    unsigned long long wait_ns;   // limit of a wait for the previous sweep
     unsigned* bar;                // [2 * DW_MAX_RHS]: barrier and exit counts per rhs (left at zero)
     int* err_host;
 };
@@ -298,8 +300,8 @@ __device__ __forceinline__ void cta_sum3(C& a, C& b, C& c, C* red) {
     }
 }
 
-// waits until *cnt reaches target, giving up after about two seconds
-__device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target) {
+// waits until *cnt reaches target, giving up after limit ns
+__device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target, unsigned long long limit) {
     unsigned long long t0 = 0;
     for (unsigned it = 1;; ++it) {
         unsigned v;
@@ -309,7 +311,7 @@ __device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target)
             const unsigned long long now = global_ns();
             if (t0 == 0)
                 t0 = now;
-            else if (now - t0 > 2000000000ULL)
+            else if (now - t0 > limit)
                 return false;
         }
     }
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
         // the previous sweep's sends have arrived: fetch the inbox
         bool ok = true;
         if (sw > a.s0) {
-            if (tid == 0) ok = count_wait(a.bar + r, ncta * (unsigned)(sw - a.s0));
+            if (tid == 0) ok = count_wait(a.bar + r, ncta * (unsigned)(sw - a.s0), a.wait_ns);
             __syncthreads();
         }
         if (sw > 0) {
@@ -700,6 +702,9 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     a.nmr = nmr;
     a.nsweeps = 2 * ncycles;
     a.clov = cl ? ((sizeof(C) == 4) ? cl->a32 : cl->a64) : nullptr;
+    // two seconds, and more than an MR step takes in any precision (70 us in FP64)
+    // for each of the steps by which another domain may be behind
+    a.wait_ns = 2000000000ULL + 200000ULL * (unsigned long long)nmr;
     a.bar = w.bar;
     a.err_host = w.err;
     cudaLaunchConfig_t cfg = {};
@@ -714,11 +719,16 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     if ((long long)cfg.gridDim.x <= fit) {
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
-        a.s0 = 0;
-        a.s1 = a.nsweeps;
-        ProfScope ps(prof, "sap_sweep", 2.0 * bytes_first + (a.nsweeps - 2) * bytes_next, a.nsweeps);
-        DW_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
-        DW_LAUNCH_CHECK();
+        // at most 256 sweeps a launch: the barrier's counter stays small and no
+        // launch holds the device for long, however many cycles are asked for
+        for (int sw = 0; sw < a.nsweeps; sw = a.s1) {
+            a.s0 = sw;
+            a.s1 = std::min(a.nsweeps, sw + 256);
+            const double bytes = (sw ? 0.0 : 2.0 * (bytes_first - bytes_next)) + (a.s1 - a.s0) * bytes_next;
+            ProfScope ps(prof, "sap_sweep", bytes, a.s1 - a.s0);
+            DW_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
+            DW_LAUNCH_CHECK();
+        }
         return DW_OK;
     }
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

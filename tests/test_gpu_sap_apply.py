@@ -29,8 +29,12 @@ CASES = [
 ]
 
 
-@pytest.mark.parametrize("prec", ["f64", "f32", "f16", "bf16"])
-@pytest.mark.parametrize("dims,block,cycles,mr,nrhs,csw", CASES)
+# 260 sweeps: more than one cooperative launch takes
+LONG = ((4, 4, 4, 4), (2, 2, 2, 2), 130, 1, 1, 0.0)
+
+
+@pytest.mark.parametrize("dims,block,cycles,mr,nrhs,csw,prec",
+                         [c + (p,) for c in CASES for p in TOL] + [LONG + ("f64",)])
 def test_sap_matches_oracle(dims, block, cycles, mr, nrhs, csw, prec):
     import paper_1204_5463_gb300 as dw
 
