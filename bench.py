@@ -137,9 +137,9 @@ def kernel_traffic(name):
 
 def dw_bandwidth(peaks, reps=10, dims=(24, 24, 24, 48)):
     """The full-lattice stencil alone on a 24^3 x 48 lattice by default (its
-    links and fields, 318 MB in FP32, exceed L2): algorithmic bytes per site (links +
-    input + output: 960 B FP64, 480 B FP32, 248 B FP16 with scales) over the
-    kernel's CUDA-event time, per storage precision. L2 is flushed (a 256 MB
+    links and fields, 382 MB in FP32, exceed L2): algorithmic bytes per site (links,
+    input in storage format, output in the caller's FP64 layout: 960 B FP64, 576 B
+    FP32, 388 B FP16 with scales) over the kernel's CUDA-event time, per storage precision. L2 is flushed (a 256 MB
     write) before every call; each call converts its input to the internal
     layout right before the stencil, so part of that input can still be in L2."""
     import numpy as np
@@ -479,8 +479,7 @@ def _profiled_sap(dw, torch, ctx, bd, ncyc, nmr, prec, nrhs, V, block):
     avg_s = d["total_ms"] / d["launches"] / 1e3
     flops = nrhs * (V / 2) * sap_flops_per_site(block, nmr)
     tf = flops / avg_s / 1e12
-    # whole applications without per-kernel events (consecutive sweeps keep
-    # their programmatic overlap): time per sweep, conversions included
+    # whole applications without per-kernel events: time per sweep, conversions included
     st = torch.cuda.current_stream()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record(st)

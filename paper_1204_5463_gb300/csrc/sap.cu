@@ -1,5 +1,7 @@
 // One colour half-sweep of the Schwarz alternating procedure (Sec. 2,
 // Algorithm 2) with inexact minimal-residual domain solves (Sec. 4).
+// For the domains that sap_apply.cu does not take (more than 256 sites, or a
+// halo above 192 bytes a site): that form is faster wherever it fits.
 //
 // One CTA owns one domain L^l of the swept colour (and one right-hand side);
 // one thread owns one site of the domain. The CTA
