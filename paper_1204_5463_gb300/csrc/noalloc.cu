@@ -3,7 +3,7 @@
 // allocate device memory -- code running inside a pre-reserved memory pool,
 // under an allocator that forbids cudaMalloc, or in a process whose memory
 // budget is fixed at start-up. The internal-layout copies of the links and of
-// the input/output fields live in one file-scope __device__ array instead of
+// the input field live in one file-scope __device__ array instead of
 // buffers of a context.
 #include <map>
 #include <mutex>
@@ -12,8 +12,9 @@
 
 namespace {
 
-// 480 bytes per site (FP32 links 288 + input 96 + output 96) for up to 4096
-// sites. Every device that loads the library holds this array until exit.
+// 480 bytes per site for up to 4096 sites, the documented footprint (FP32 links
+// 288 and input 96; the stencil writes its output to the caller itself). Every
+// device that loads the library holds this array until exit.
 constexpr long long kNoAllocMaxSites = 4096;
 constexpr size_t kNoAllocBytes = 480 * kNoAllocMaxSites;
 static __device__ __align__(256) unsigned char g_dw_noalloc_scratch[kNoAllocBytes];
