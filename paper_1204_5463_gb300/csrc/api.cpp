@@ -180,16 +180,14 @@ static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** 
     return DW_OK;
 }
 
-int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
-            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
+int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* state, long long state_rs,
+            char* inbox, long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
     const Geom& g = ctx->g;
     const long long sb = spinor_bytes(prec, g.V);
     const double first = 0.5 * ((double)nact * 2.0 * sb + link_bytes(prec, g.V));
     const double next = 0.5 * ((double)nact * 3.0 * sb + link_bytes(prec, g.V));
-    const char *U, *Uimg;
     int rc;
     if (sap_apply_fits(prec, g)) {
-        if ((rc = sap_links_for(ctx, prec, 0, &U, &Uimg))) return rc;
         SapWork w;
         w.Uimg = Uimg;
         w.rho = state;
@@ -203,7 +201,6 @@ int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long lon
                                 &ctx->prof, first, next);
     }
     const int thr = ctx->sap_threads[prec];
-    if ((rc = sap_links_for(ctx, prec, thr, &U, &Uimg))) return rc;
     for (int cyc = 0; cyc < ncycles; ++cyc)
         for (int colour = 0; colour < 2; ++colour) {
             const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
@@ -369,6 +366,9 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     const long long V = ctx->g.V;
     const long long fb = spinor_bytes(storage, V);
     int rc;
+    const char *U, *Uimg;
+    // the image is packed before the conversion's launch, not right before the sweeps (sap_run)
+    if ((rc = sap_links_for(ctx, storage, ctx->sap_threads[storage], &U, &Uimg))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = ctx->work_out.ensure((size_t)nrhs * fb))) return rc;
     const size_t sbytes = sap_state_bytes(storage, ctx->g), ibytes = sap_inbox_bytes(storage, ctx->g);
@@ -376,7 +376,7 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     char* scratch = ctx->work_sap.as<char>();
     if ((rc = launch_to_internal(storage, v, ctx->work_in.as<char>(), V, nrhs, ctx->stream))) return rc;
     FieldRef fv{ctx->work_in.as<char>(), fb, 0, 0}, fx{ctx->work_out.as<char>(), fb, 0, 0};
-    if ((rc = sap_run(ctx, storage, fv, fx, scratch, (long long)sbytes, scratch + nrhs * sbytes, (long long)ibytes,
+    if ((rc = sap_run(ctx, storage, Uimg, fv, fx, scratch, (long long)sbytes, scratch + nrhs * sbytes, (long long)ibytes,
                       nullptr, nrhs, nrhs, ncycles, nmr)))
         return rc;
     if ((rc = launch_from_internal(storage, ctx->work_out.as<char>(), z, V, nrhs, ctx->stream))) return rc;

@@ -224,9 +224,13 @@ size_t sap_state_bytes(int prec, const Geom& g);
 size_t sap_inbox_bytes(int prec, const Geom& g);
 // the whole application, nact of the nrhs right-hand sides active: by
 // launch_sap_apply where the domain fits, else sweep by sweep (the scratch is
-// then unused); state and inbox: scratch of the strides given
-int sap_run(dw_ctx* ctx, int prec, FieldRef v, FieldRef x, char* state, long long state_rs, char* inbox,
-            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
+// then unused); state and inbox: scratch of the strides given. Uimg: the image
+// of sap_links_for, packed (if it had to be) before at least one ordinary launch
+// or copy of the stream: the first sweep is launched programmatically and reads the
+// image before it waits for the kernel in front of it, so that kernel must not
+// be the one that writes the image.
+int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* state, long long state_rs,
+            char* inbox, long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
 // after the stream was synchronised: DW_ETIMEOUT if a SAP kernel's bounded wait gave up
 int sap_check(dw_ctx* ctx);
 

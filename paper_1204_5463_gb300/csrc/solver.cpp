@@ -95,7 +95,7 @@ struct Solver {
     long long fv;       // bytes of one basis vector in format vp
     int NP;             // multi-dot row length (m + 2)
     int nblk;
-    const char *U_mv, *U64;
+    const char *U_sap_img, *U_mv, *U64;
     // device buffers (owned by the workspace of the context)
     char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap, *canon;
     double2 *partial, *dots, *Qd, *etad;
@@ -214,7 +214,7 @@ int Solver::setup() {
     NP = m + 2;
     nblk = blas_nblk(n);
     int rc;
-    const char *U_sap, *U_sap_img;  // the preconditioner's links, before the first step needs them
+    const char* U_sap;
     if ((rc = sap_links_for(ctx, sp, ctx->sap_threads[sp], &U_sap, &U_sap_img))) return rc;
     if ((rc = gauge_for(ctx, mp == P64 ? P64 : P32, &U_mv))) return rc;
     // explicit residual: FP64 links for FP64 outer vectors, double-float links otherwise
@@ -506,7 +506,7 @@ int Solver::step() {
     // The preconditioner's scratch lies in rb (the explicit residual is formed
     // and consumed within cycle_end, so rb is free during the steps) and in the
     // staging copy of the right-hand sides: 192 bytes per site and rhs each.
-    if ((rc = sap_run(ctx, sp, Lf, Zs, rb, fb, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
+    if ((rc = sap_run(ctx, sp, U_sap_img, Lf, Zs, rb, fb, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
         return rc;
     if (zp != sp) {
         ProfScope ps(&ctx->prof, "z_widen", (double)nact * (sb + zb));
