@@ -115,9 +115,8 @@ int dw_apply(dw_ctx* ctx, const double* in, double* out, dw_prec prec, int nrhs)
 /* z = M v with M the SAP preconditioner (Sec. 4): ncycles iterations of
  * Algorithm 2 started from x = 0, each a sweep over the domains of colour 0
  * (block coordinates summing to an even number; contains site 0) followed by
- * colour 1. Each domain solve starts from r = (v - D x)^l of the full
- * operator (carried from visit to visit with the neighbours' corrections, or
- * recomputed for domains whose halo does not fit), runs nmr minimal-residual
+ * colour 1. Each domain solve computes r = (v - D x)^l with the full
+ * operator (x as the storage precision holds it), runs nmr minimal-residual
  * steps on D^l y = r from y = 0 (Sec. 4) and adds x^l += y^l. storage selects the precision of v, x and the links
  * (arithmetic FP32 for DW_F32/F16/BF16, FP64 for DW_F64).
  * v, z: device pointers, canonical FP64 layout, nrhs fields each.

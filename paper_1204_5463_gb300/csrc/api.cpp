@@ -180,8 +180,8 @@ static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** 
     return DW_OK;
 }
 
-int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* state, long long state_rs,
-            char* inbox, long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
+int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* inbox,
+            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
     const Geom& g = ctx->g;
     const long long sb = spinor_bytes(prec, g.V);
     const double first = 0.5 * ((double)nact * 2.0 * sb + link_bytes(prec, g.V));
@@ -190,9 +190,6 @@ int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, cha
     if (sap_apply_fits(prec, g)) {
         SapWork w;
         w.Uimg = Uimg;
-        w.rho = state;
-        w.rho_rs = w.xpart_rs = state_rs;
-        w.xpart = state + spinor_bytes(P32, g.V);
         w.inbox = inbox;
         w.inbox_rs = inbox_rs;
         w.err = ctx->sap_err.d;
@@ -371,13 +368,12 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     if ((rc = sap_links_for(ctx, storage, ctx->sap_threads[storage], &U, &Uimg))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = ctx->work_out.ensure((size_t)nrhs * fb))) return rc;
-    const size_t sbytes = sap_state_bytes(storage, ctx->g), ibytes = sap_inbox_bytes(storage, ctx->g);
-    if (sap_apply_fits(storage, ctx->g) && (rc = ctx->work_sap.ensure((size_t)nrhs * (sbytes + ibytes)))) return rc;
-    char* scratch = ctx->work_sap.as<char>();
+    const size_t ibytes = sap_inbox_bytes(storage, ctx->g);
+    if (sap_apply_fits(storage, ctx->g) && (rc = ctx->work_sap.ensure((size_t)nrhs * ibytes))) return rc;
     if ((rc = launch_to_internal(storage, v, ctx->work_in.as<char>(), V, nrhs, ctx->stream))) return rc;
     FieldRef fv{ctx->work_in.as<char>(), fb, 0, 0}, fx{ctx->work_out.as<char>(), fb, 0, 0};
-    if ((rc = sap_run(ctx, storage, Uimg, fv, fx, scratch, (long long)sbytes, scratch + nrhs * sbytes, (long long)ibytes,
-                      nullptr, nrhs, nrhs, ncycles, nmr)))
+    if ((rc = sap_run(ctx, storage, Uimg, fv, fx, ctx->work_sap.as<char>(), (long long)ibytes, nullptr, nrhs, nrhs,
+                      ncycles, nmr)))
         return rc;
     if ((rc = launch_from_internal(storage, ctx->work_out.as<char>(), z, V, nrhs, ctx->stream))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));

@@ -288,17 +288,20 @@ __device__ __forceinline__ uint32_t f2_to_h2(float a, float b, int bf) {
     return u;
 }
 
-template <class T, bool G>
+template <class T, int G>
 __device__ __forceinline__ T ld(const T* p) {
-    if constexpr (G)
+    if constexpr (G == 2)
+        return __ldcg(p);
+    else if constexpr (G == 1)
         return __ldg(p);
     else
         return *p;
 }
 
 // load the 12 complex components of site s into compute type C
-// (G = true: global memory through the read-only path; false: shared memory)
-template <int P, class C, bool G = true>
+// (G = 1: global memory through the read-only path; 2: through L2, for what the
+// same kernel wrote; 0: shared memory)
+template <int P, class C, int G = 1>
 __device__ __forceinline__ void load_spinor(const char* base, long long V, long long s, cx<C> out[12]) {
     if constexpr (P == PDF && std::is_same<C, df>::value) {
         const float4* p = reinterpret_cast<const float4*>(base);

@@ -197,15 +197,13 @@ int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, in
 // (the image is packed on first use and after dw_set_gauge), and the error flag
 int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char** img);
 // ----- sap_apply.cu --------------------------------------------------------
-// z = M v with the domains' residuals carried along (sap_apply.cu), for
-// domains that sap_apply_fits accepts. Per right-hand side: rho (the residuals,
-// spinor layout of the arithmetic precision), xpart (the same size, only for
-// 16-bit storage) and the inboxes.
+// z = M v with the domains' halos exchanged as half spinors (sap_apply.cu), for
+// domains that sap_apply_fits accepts. inbox: scratch per right-hand side.
 struct SapWork {
     const char* Uimg;
     const unsigned short* faces;
-    char *rho, *xpart, *inbox;
-    long long rho_rs, xpart_rs, inbox_rs;
+    char* inbox;
+    long long inbox_rs;
     unsigned* bar;
     int* err;
 };
@@ -217,20 +215,18 @@ int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st);
 int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab,
                      int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
                      double bytes_first, double bytes_next);
-// Scratch of one application and right-hand side in two pieces: the residuals
-// (with the 16-bit formats' iterate behind them) and the inboxes. Neither
-// exceeds a double-precision field (192 bytes per site).
-size_t sap_state_bytes(int prec, const Geom& g);
+// Scratch of one application and right-hand side: at most a double-precision
+// field (192 bytes per site).
 size_t sap_inbox_bytes(int prec, const Geom& g);
 // the whole application, nact of the nrhs right-hand sides active: by
 // launch_sap_apply where the domain fits, else sweep by sweep (the scratch is
-// then unused); state and inbox: scratch of the strides given. Uimg: the image
+// then unused); inbox: scratch of the stride given. Uimg: the image
 // of sap_links_for, packed (if it had to be) before at least one ordinary launch
 // or copy of the stream: the first sweep is launched programmatically and reads the
 // image before it waits for the kernel in front of it, so that kernel must not
 // be the one that writes the image.
-int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* state, long long state_rs,
-            char* inbox, long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
+int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* inbox,
+            long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
 // after the stream was synchronised: DW_ETIMEOUT if a SAP kernel's bounded wait gave up
 int sap_check(dw_ctx* ctx);
 

@@ -1,18 +1,22 @@
-// The SAP preconditioner z = M v (Sec. 2, Algorithm 2; Sec. 4) with the residual
-// carried along instead of recomputed.
+// The SAP preconditioner z = M v (Sec. 2, Algorithm 2; Sec. 4) with the domains'
+// halos exchanged as half spinors.
 //
-// Algorithm 2 takes, for every domain it sweeps, r^l = (v - D x)^l. Between two
-// visits of a domain only its neighbours' iterates change, so
-//   r^l = rho^l + 1/2 sum over the hops that enter L^l of the neighbours' last
-//         corrections y,
-// where rho^l is the residual that the domain's own MR solve left. A domain
-// therefore keeps rho^l, and after its solve sends one spin-projected half
-// spinor per face site and direction to the neighbouring domains' inboxes:
-//   to the domain one step down in mu:  (1 + gamma_mu) y   (upper two rows; the
+// Every sweep takes, for each domain of its colour, r^l = (v - D x)^l, solves D^l y
+// = r^l by MR steps and adds y to x^l. After its solve a domain sends one
+// spin-projected half spinor of its new x, rounded as storage holds it, per face
+// site and direction to the neighbouring domains' inboxes:
+//   to the domain one step down in mu:  (1 + gamma_mu) x   (upper two rows; the
 //       receiver owns the link and multiplies by U),
-//   to the domain one step up in mu:    U^dagger (1 - gamma_mu) y.
-// An inbox is contiguous, so a domain fetches its whole halo with coalesced
-// 16-byte copies and the residual costs only the hops that cross its faces.
+//   to the domain one step up in mu:    U^dagger (1 - gamma_mu) x.
+// An inbox is contiguous, its slots in the order of a face's sites: the sites of a
+// face read it through L2 in whole lines, half the bytes of a spinor and no link.
+// The hops inside the domain come from the domain's own x in shared memory. x, in
+// storage format, is all that is kept between sweeps. (The residual that the MR
+// solve leaves could be carried along instead, with half spinors of y: a local
+// stencil less a sweep, 298 us instead of 314 in the first line of the table below,
+// 11.4 ms instead of 13.4 in its fourth. But the rounding of x then never enters r:
+// FP32 errors of 1.8e-7 instead of 1.5e-7, and residuals of 4 u instead of 1.3 u
+// after many cycles.)
 //
 // One CTA owns one domain (and right-hand side), one thread one site. Sweeps
 // either run as one launch each, or, when the domains of one colour and all
@@ -20,18 +24,19 @@
 // barrier per right-hand side between sweeps: the CTA then fetches the links
 // of its next domain while the barrier completes.
 //
-// What it replaces and what bounds it: recomputing r costs every sweep the full
-// stencil (1392 flop a site), whose halo reads leave L2 one hop at a time
-// (5.3 us of a 22 us sweep), and a launch per sweep costs 8-9 us between the
-// sweeps of 256 domains. Here the residual takes 1.8 us, and the sends 1.2 us.
-// Measured against one launch of sap_sweep_kernel per sweep (5 cycles x 4 MR
-// steps unless stated): 8^3 x 16, 2 rhs served on 4 streams 38.2 -> 28.8 ms a
-// burst; 12^3 x 18 in 3^4 domains, 3 BF16 rhs (4 x 5) 341 -> 279 us; 24^3 x 48,
-// 12 FP16 rhs 14.91 -> 12.48 ms; 16^3 x 32 FP32 342 -> 302 us, with the clover
-// term (8 x 5) 766 -> 630 us. Four fifths of that are the MR steps, bound by the
-// latency of shared memory at the 16 warps that 128 registers allow, with its
-// pipe busy three quarters of the time; paired, scalar and mixed forms of the
-// hop's FP32 arithmetic are within 2% of one another.
+// What it replaces and what bounds it: sap_sweep_kernel reads the spinors and links
+// of the halo from L2 one hop at a time (5.3 us of a 22 us sweep), and a launch per
+// sweep costs 8-9 us between the sweeps of 256 domains. Its results are the
+// same to the bit (in FP64 up to rounding). Calls, conversions included (5 cycles x 4 MR steps unless stated):
+//   16^3 x 32, 4^4 domains, FP32                 343 -> 314 us
+//   the same with the clover term (8 x 5)        759 -> 719 us
+//   12^3 x 18, 3^4 domains, 3 BF16 rhs (4 x 5)   342 -> 284 us
+//   24^3 x 48, 4^4 domains, 12 FP16 rhs         14.93 -> 13.38 ms
+//   8^3 x 16, 2 rhs, solves on 4 streams         38.2 -> 28.7 ms a burst
+// Three quarters are the MR steps, bound by the latency of shared memory at the 16
+// warps that 128 registers allow, with its pipe busy three quarters of the time;
+// paired, scalar and mixed forms of the hop's FP32 arithmetic are within 2% of one
+// another.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -53,10 +58,6 @@ struct SapArgs {
     const char* Uimg;             // links of every domain as the shared-memory image of LinkWarp
     const unsigned short* faces;  // [ns / 2]: lower-face site | mu << 10 of an inbox slot
     int ns;                       // inbox slots per domain (two per face site and direction)
-    char* rho;                    // per rhs: the domains' residuals, site layout of the arithmetic type
-    long long rho_rs;
-    char* xpart;                  // per rhs: the iterate between cycles, same layout
-    long long xpart_rs;
     char* inbox;                  // per rhs: [domain] of Half<C> boxes
     long long inbox_rs;
     RhsCols jtab;
@@ -68,33 +69,11 @@ struct SapArgs {
     int* err_host;
 };
 
-// a site's spinor in the layout of S32 / S64, read through L2 (other SMs wrote it)
-template <class C>
-__device__ __forceinline__ void state_load(const char* base, long long V, long long s, cx<C> out[12]) {
-    if constexpr (sizeof(C) == 4) {
-        const float4* p = reinterpret_cast<const float4*>(base);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const float4 v = __ldcg(&p[q * V + s]);
-            out[2 * q] = mk<C>(v.x, v.y);
-            out[2 * q + 1] = mk<C>(v.z, v.w);
-        }
-    } else {
-        const double2* p = reinterpret_cast<const double2*>(base);
-#pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const double2 v = __ldcg(&p[c * V + s]);
-            out[c] = mk<C>(v.x, v.y);
-        }
-    }
-}
-
-// Shared-memory layouts in pieces of a warp's 32 sites (inbox: of 8 slots), so that
-// every plane lies at a compile-time offset from one address: with planes of T
+// Shared-memory layouts in pieces of a warp's 32 sites, so that every plane lies at a compile-time offset from one address: with planes of T
 // sites each load had its own address arithmetic, a sixth of an MR step's
 // instructions.
 //
-// The site vectors rho and y: FP32 float4 [warp][6][32], FP64 double2 [warp][12][32].
+// The site vectors x and rho: FP32 float4 [warp][6][32], FP64 double2 [warp][12][32].
 template <class C>
 struct SiteVec {
     static constexpr int kPlanes = sizeof(C) == 4 ? 6 : 12;
@@ -183,7 +162,8 @@ struct LinkWarp {
     }
 };
 
-// Half spinors (the upper two spin rows), in boxes of 8 slots: 16-byte words [3 or 6][8]
+// Half spinors (the upper two spin rows) of an inbox in global memory, in boxes of 8
+// slots: 16-byte words [3 or 6][8], read through L2 (other SMs write them)
 template <class C>
 struct Half {
     static constexpr int kWords = sizeof(C) == 4 ? 3 : 6;
@@ -192,15 +172,15 @@ struct Half {
     static __device__ __forceinline__ int at(int q) { return (q >> 3) * kBox + (q & 7) * 16; }
     static __device__ __forceinline__ void load(const unsigned char* p, cx<C> h0[3], cx<C> h1[3]) {
         if constexpr (sizeof(C) == 4) {
-            const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 128),
-                         c = *reinterpret_cast<const float4*>(p + 256);
+            const float4* w = reinterpret_cast<const float4*>(p);
+            const float4 a = __ldcg(w), b = __ldcg(w + 8), c = __ldcg(w + 16);
             h0[0] = mk<C>(a.x, a.y), h0[1] = mk<C>(a.z, a.w), h0[2] = mk<C>(b.x, b.y);
             h1[0] = mk<C>(b.z, b.w), h1[1] = mk<C>(c.x, c.y), h1[2] = mk<C>(c.z, c.w);
         } else {
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const double2 a = *reinterpret_cast<const double2*>(p + 128 * i),
-                              b = *reinterpret_cast<const double2*>(p + 128 * (3 + i));
+                const double2* w = reinterpret_cast<const double2*>(p) + 8 * i;
+                const double2 a = __ldcg(w), b = __ldcg(w + 24);
                 h0[i] = mk<C>(a.x, a.y);
                 h1[i] = mk<C>(b.x, b.y);
             }
@@ -221,16 +201,16 @@ struct Half {
     }
 };
 
-// what a face site sends: SIDE 0, its lower face: (1 + gamma_MU) y; SIDE 1,
-// its upper face: U^dagger (1 - gamma_MU) y
+// what a face site sends: SIDE 0, its lower face: (1 + gamma_MU) x; SIDE 1,
+// its upper face: U^dagger (1 - gamma_MU) x
 template <int MU, class C, class LW>
-__device__ __forceinline__ void face_half(int side, const cx<C> y[12], const unsigned char* lsh, int t, cx<C> k0[3],
+__device__ __forceinline__ void face_half(int side, const cx<C> x[12], const unsigned char* lsh, int t, cx<C> k0[3],
                                           cx<C> k1[3]) {
     if (side == 0) {
-        project<MU, +1, C>(y, k0, k1);
+        project<MU, +1, C>(x, k0, k1);
     } else {
         cx<C> h0[3], h1[3], u[9];
-        project<MU, -1, C>(y, h0, h1);
+        project<MU, -1, C>(x, h0, h1);
         LW::template load<C>(lsh, MU, t, u);
         su3_mul<C, true, kChain>(u, h0, k0);
         su3_mul<C, true, kChain>(u, h1, k1);
@@ -272,8 +252,8 @@ __device__ __forceinline__ void hop_if(bool in, const cx<C> psi[12], const cx<C>
 }
 
 // CTA-wide sums of three numbers, at most 8 warps: within a warp the three
-// are folded together (lanes end up with one number each), across warps every
-// lane adds one warp's numbers. red: [8][4].
+// are folded together (lanes end up with one number each), then every thread adds
+// the warps' sums in order. red: [8][4].
 template <class C>
 __device__ __forceinline__ void cta_sum3(C& a, C& b, C& c, C* red) {
     constexpr unsigned full = 0xffffffffu;
@@ -287,16 +267,11 @@ __device__ __forceinline__ void cta_sum3(C& a, C& b, C& c, C* red) {
     for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(full, k, o);
     if ((lane & 7) == 0) red[4 * (threadIdx.x >> 5) + (lane >> 3)] = k;
     __syncthreads();
-    const int w = lane & 7;
-    const bool on = w < nw;
-    a = on ? red[4 * w] : C(0);
-    b = on ? red[4 * w + 1] : C(0);
-    c = on ? red[4 * w + 2] : C(0);
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(full, a, o);
-        b += __shfl_xor_sync(full, b, o);
-        c += __shfl_xor_sync(full, c, o);
+    a = b = c = C(0);
+    for (int w = 0; w < nw; ++w) {
+        a += red[4 * w];
+        b += red[4 * w + 1];
+        c += red[4 * w + 2];
     }
 }
 
@@ -319,16 +294,16 @@ __device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target,
 
 template <int PS, int PL, class C, bool CLOV>
 __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(const __grid_constant__ SapArgs<C> a) {
-    constexpr int CP = (sizeof(C) == 4) ? P32 : P64;  // layout of rho and xpart, storage of the clover term
+    constexpr int CP = (sizeof(C) == 4) ? P32 : P64;  // storage of the clover term
     typedef LinkWarp<PL> LW;
     typedef SiteVec<C> SV;
     typedef Half<C> HB;
     extern __shared__ __align__(16) unsigned char smem[];
     const Geom& g = a.g;
     const int T = blockDim.x, ns = a.ns, hbytes = HB::bytes(ns);
-    unsigned char* rsh = smem;                                          // inbox, then rho, then y
-    unsigned char* lsh = smem + max(SV::kWarp * (T >> 5), hbytes);      // links
-    C* red = reinterpret_cast<C*>(lsh + LW::kWarp * (T >> 5));          // [8][4]
+    unsigned char* rsh = smem;                                  // x, then rho, then the new x
+    unsigned char* lsh = smem + SV::kWarp * (T >> 5);           // links
+    C* red = reinterpret_cast<C*>(lsh + LW::kWarp * (T >> 5));  // [8][4]
     unsigned long long* lbar = reinterpret_cast<unsigned long long*>(red + 32);
 
     const int r = blockIdx.x % a.nrhs;
@@ -336,8 +311,6 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
     if (!rhs_active(a.jtab, r)) return;  // every CTA of this rhs
     const char* vb = field_ptr(a.v, a.jtab, r);
     char* xb = field_ptr(a.x, a.jtab, r);
-    char* rho_g = a.rho + (long long)r * a.rho_rs;
-    char* xp = (PS == P16 || PS == PB16) ? a.xpart + (long long)r * a.xpart_rs : xb;
     unsigned char* inb = reinterpret_cast<unsigned char*>(a.inbox) + (long long)r * a.inbox_rs;
     const unsigned ncta = (unsigned)g.ndom / 2;  // CTAs of this rhs
 
@@ -393,10 +366,15 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();  // the mbarrier is initialised before any thread waits on it
 
-    const C m2diag = -2 * a.diag;
+    const C diag2 = 2 * a.diag;
+    // inbox slots of this site's lines in the four directions
+    const int q0 = lx[1] + g.b[1] * (lx[2] + g.b[2] * lx[3]);
+    const int q1 = g.B / g.b[0] + lx[0] + g.b[0] * (lx[2] + g.b[2] * lx[3]);
+    const int q2 = g.B / g.b[0] + g.B / g.b[1] + lx[0] + g.b[0] * (lx[1] + g.b[1] * lx[3]);
+    const int q3 = g.B / g.b[0] + g.B / g.b[1] + g.B / g.b[2] + lx[0] + g.b[0] * (lx[1] + g.b[1] * lx[2]);
     bool dead = false;
     for (int sw = a.s0; sw < a.s1; ++sw) {
-        const bool first = sw < 2, last = sw >= a.nsweeps - 2;
+        const bool first = sw < 2;  // x^l is still zero
         long long s;
         {
             int xg[4];
@@ -407,26 +385,22 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
             s = site_index(g, xg);
         }
         cx<C> rho[12], y[12];
+        // the domain's own iterate (written by this thread two sweeps ago) and v
         if (act) {
-            if (first)
-                load_spinor<PS, C>(vb, g.V, s, rho);
-            else
-                state_load<C>(rho_g, g.V, s, rho);
+            if (!first) {
+                load_spinor<PS, C, 2>(xb, g.V, s, y);
+                SV::store(own, y);
+            }
+            if (sw == 0) load_spinor<PS, C>(vb, g.V, s, rho);
         } else {
 #pragma unroll
             for (int c = 0; c < 12; ++c) rho[c] = czero<C>();
         }
-        // the previous sweep's sends have arrived: fetch the inbox
+        // the previous sweep's sends have arrived
         bool ok = true;
         if (sw > a.s0) {
             if (tid == 0) ok = count_wait(a.bar + r, ncta * (unsigned)(sw - a.s0), a.wait_ns);
             __syncthreads();
-        }
-        if (sw > 0) {
-            const unsigned char* src = inb + (long long)dom * hbytes;
-            for (int q = tid; q < hbytes / 16; q += T)
-                cp_async_word(reinterpret_cast<float4*>(rsh) + q, reinterpret_cast<const float4*>(src) + q);
-            cp_async_wait();
         }
         ok = ok && bulk_copy_wait(lbar, (sw - a.s0) & 1);
         if (__syncthreads_or(!ok)) {
@@ -438,62 +412,103 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
             dead = true;
             break;
         }
-        // r = rho + 1/2 sum of the hops that enter the domain: first the link
-        // products of the forward half spinors, one face site per thread, in place ...
-        if (sw > 0) {
-            for (int q = tid; q < ns / 2; q += T) {
-                const int f = __ldg(a.faces + q), mu = f >> 10;
-                const int t = (f & 1023) + (mu == 0 ? g.b[0] - 1 : mu == 1 ? (g.b[1] - 1) * ls1
-                                            : mu == 2       ? (g.b[2] - 1) * ls2
-                                                            : (g.b[3] - 1) * ls3);
-                cx<C> h0[3], h1[3], k0[3], k1[3], u[9];
-                HB::load(rsh + HB::at(q), h0, h1);
-                LW::template load<C>(lsh, mu, t, u);
-                su3_mul<C, false, kChain>(u, h0, k0);
-                su3_mul<C, false, kChain>(u, h1, k1);
-                HB::store(rsh + HB::at(q), k0, k1);
-            }
-            __syncthreads();
-            // ... then each site adds what enters through its faces
-            if (act) {
-                cx<C> acc[12], k0[3], k1[3];
+        // r = v - D x at this site: neighbours inside the domain from shared memory,
+        // the others' half spinors from the inbox (fetched one direction ahead)
+        if (act && sw > 0) {
+            cx<C> acc[12], e0[3], e1[3];
 #pragma unroll
-                for (int c = 0; c < 12; ++c) acc[c] = czero<C>();
-                int off = 0;  // slot of this site's line in direction mu
-#define SAP_IN_HOPS(MU, FI)                                     \
-    {                                                           \
-        const int q = off + (FI);                               \
-        if (lx[MU] == g.b[MU] - 1) {                            \
-            HB::load(rsh + HB::at(q), k0, k1);                  \
-            reconstruct<MU, +1, C>(k0, k1, acc);                \
-        }                                                       \
-        if (lx[MU] == 0) {                                      \
-            HB::load(rsh + HB::at(ns / 2 + q), k0, k1);         \
-            reconstruct<MU, -1, C>(k0, k1, acc);                \
-        }                                                       \
-        off += g.B / g.b[MU];                                   \
+            for (int c = 0; c < 12; ++c) acc[c] = czero<C>();
+            const unsigned char* box = inb + (long long)dom * hbytes;
+#define SAP_FETCH(MU)                                                                        \
+    {                                                                                        \
+        if (lx[MU] + 1 == g.b[MU])                                                           \
+            HB::load(box + HB::at(q##MU), e0, e1);                                           \
+        else if (lx[MU] == 0)                                                                \
+            HB::load(box + HB::at(ns / 2 + q##MU), e0, e1);                                  \
     }
-                SAP_IN_HOPS(0, lx[1] + g.b[1] * (lx[2] + g.b[2] * lx[3]))
-                SAP_IN_HOPS(1, lx[0] + g.b[0] * (lx[2] + g.b[2] * lx[3]))
-                SAP_IN_HOPS(2, lx[0] + g.b[0] * (lx[1] + g.b[1] * lx[3]))
-                SAP_IN_HOPS(3, lx[0] + g.b[0] * (lx[1] + g.b[1] * lx[2]))
+#define SAP_RES_HOPS(MU, LS_MU, NEXT)                                                        \
+    {                                                                                        \
+        const bool up = lx[MU] + 1 < g.b[MU], dn = lx[MU] >= 1;                              \
+        cx<C> psi[12], u[9], h0[3], h1[3], k0[3], k1[3], f0[3], f1[3];                       \
+        _Pragma("unroll") for (int c = 0; c < 3; ++c) f0[c] = e0[c], f1[c] = e1[c];          \
+        NEXT;                                                                                \
+        SV::load(rsh + SV::at(up ? tid + LS_MU : tid), psi);                                 \
+        project<MU, +1, C>(psi, h0, h1);                                                     \
+        _Pragma("unroll") for (int c = 0; c < 3; ++c) {                                      \
+            h0[c] = up ? h0[c] : f0[c];                                                      \
+            h1[c] = up ? h1[c] : f1[c];                                                      \
+        }                                                                                    \
+        LW::template load<C>(lsh, MU, tid, u);                                               \
+        su3_mul<C, false, kChain>(u, h0, k0);                                                \
+        su3_mul<C, false, kChain>(u, h1, k1);                                                \
+        reconstruct<MU, +1, C>(k0, k1, acc);                                                 \
+        if (!up && !dn) HB::load(box + HB::at(ns / 2 + q##MU), f0, f1);                      \
+        const int td = dn ? tid - LS_MU : tid;                                               \
+        SV::load(rsh + SV::at(td), psi);                                                     \
+        LW::template load<C>(lsh, MU, td, u);                                                \
+        project<MU, -1, C>(psi, h0, h1);                                                     \
+        su3_mul<C, true, kChain>(u, h0, k0);                                                 \
+        su3_mul<C, true, kChain>(u, h1, k1);                                                 \
+        _Pragma("unroll") for (int c = 0; c < 3; ++c) {                                      \
+            k0[c] = dn ? k0[c] : f0[c];                                                      \
+            k1[c] = dn ? k1[c] : f1[c];                                                      \
+        }                                                                                    \
+        reconstruct<MU, -1, C>(k0, k1, acc);                                                 \
+    }
+#define SAP_IN_HOPS(MU)                                                                      \
+    {                                                                                        \
+        cx<C> u[9], h0[3], h1[3], k0[3], k1[3];                                              \
+        if (lx[MU] + 1 == g.b[MU]) {                                                         \
+            HB::load(box + HB::at(q##MU), h0, h1);                                           \
+            LW::template load<C>(lsh, MU, tid, u);                                           \
+            su3_mul<C, false, kChain>(u, h0, k0);                                            \
+            su3_mul<C, false, kChain>(u, h1, k1);                                            \
+            reconstruct<MU, +1, C>(k0, k1, acc);                                             \
+        }                                                                                    \
+        if (lx[MU] == 0) {                                                                   \
+            HB::load(box + HB::at(ns / 2 + q##MU), k0, k1);                                  \
+            reconstruct<MU, -1, C>(k0, k1, acc);                                             \
+        }                                                                                    \
+    }
+            if (first) {
+                SAP_IN_HOPS(0)
+                SAP_IN_HOPS(1)
+                SAP_IN_HOPS(2)
+                SAP_IN_HOPS(3)
+                load_spinor<PS, C>(vb, g.V, s, rho);
+            } else {
+                SAP_FETCH(0)
+                SAP_RES_HOPS(0, 1, SAP_FETCH(1))
+                SAP_RES_HOPS(1, ls1, SAP_FETCH(2))
+                SAP_RES_HOPS(2, ls2, SAP_FETCH(3))
+                load_spinor<PS, C>(vb, g.V, s, rho);
+                SAP_RES_HOPS(3, ls3, )
+            }
+#undef SAP_RES_HOPS
 #undef SAP_IN_HOPS
-                const C half = (C)0.5;
+#undef SAP_FETCH
+            const C half = (C)0.5;
+            if (first) {
 #pragma unroll
                 for (int c = 0; c < 12; ++c) rho[c] = rho[c] + half * acc[c];
+            } else {
+                SV::load(own, y);
+                if constexpr (CLOV) clover_acc<CP, C>(a.clov, g.V, s, y, acc, (C)-2);  // A x as -2 A x in acc
+#pragma unroll
+                for (int c = 0; c < 12; ++c) rho[c] = rho[c] - (a.diag * y[c] - half * acc[c]);
             }
-            __syncthreads();  // the inbox makes room for the MR iterate
         }
+        if (!first) __syncthreads();  // x makes room for the MR iterate
 #pragma unroll
         for (int c = 0; c < 12; ++c) y[c] = czero<C>();
 
-        // MR on D^l y = r^l out of shared memory, with p = -2 D^l rho:
-        // beta = <p, rho> / <p, p>, y -= 2 beta rho, rho -= beta p
+        // MR on D^l y = r^l out of shared memory, with p = 2 D^l rho:
+        // beta = <p, rho> / <p, p>, y += 2 beta rho, rho -= beta p
         for (int it = 0; it < a.nmr; ++it) {
-            cx<C> p[12];
+            cx<C> p[12];  // the hops, then p
             SV::store(own, rho);
 #pragma unroll
-            for (int c = 0; c < 12; ++c) p[c] = m2diag * rho[c];
+            for (int c = 0; c < 12; ++c) p[c] = czero<C>();
             __syncthreads();
             C pr_re = 0, pr_im = 0, pp = 0;
             if (act) {
@@ -531,39 +546,49 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
                 // neighbours read it) rather than kept in registers over the hops:
                 // the 24 registers go to overlapping the hops' loads
                 SV::load(own, rho);
-                if constexpr (CLOV) clover_acc<CP, C>(a.clov, g.V, s, rho, p, (C)-2);
+                if constexpr (CLOV) clover_acc<CP, C>(a.clov, g.V, s, rho, p, (C)-2);  // A rho as -2 A rho
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    pr_re = fma(p[c].re, rho[c].re, pr_re);
-                    pr_im = fma(p[c].re, rho[c].im, pr_im);
-                    pp = fma(p[c].re, p[c].re, pp);
-                    pr_re = fma(p[c].im, rho[c].im, pr_re);
-                    pr_im = fma(-p[c].im, rho[c].re, pr_im);
-                    pp = fma(p[c].im, p[c].im, pp);
+                    p[c] = mk<C>(fma(diag2, rho[c].re, -p[c].re), fma(diag2, rho[c].im, -p[c].im));
+                    const cx<C> t = cmulc(p[c], rho[c]);
+                    pr_re += t.re;
+                    pr_im += t.im;
+                    pp += p[c].re * p[c].re + p[c].im * p[c].im;
                 }
             }
             cta_sum3(pr_re, pr_im, pp, red);
             if (pp > (C)0) {
-                const C b_re = pr_re / pp, b_im = pr_im / pp, a_re = -2 * b_re, a_im = -2 * b_im;
+                const cx<C> beta = mk<C>(pr_re / pp, pr_im / pp), alpha = beta + beta;
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
-                    y[c].re = fma(-a_im, rho[c].im, fma(a_re, rho[c].re, y[c].re));
-                    y[c].im = fma(a_im, rho[c].re, fma(a_re, rho[c].im, y[c].im));
-                    rho[c].re = fma(b_im, p[c].im, fma(-b_re, p[c].re, rho[c].re));
-                    rho[c].im = fma(-b_im, p[c].re, fma(-b_re, p[c].im, rho[c].im));
+                    y[c] = y[c] + alpha * rho[c];
+                    rho[c] = rho[c] - beta * p[c];
                 }
             }
         }
 
-        // the correction's half spinors to the neighbouring domains' inboxes
+        // x^l <- x^l + y^l
+        if (act && !first) {
+            cx<C> xo[12];
+            load_spinor<PS, C, 2>(xb, g.V, s, xo);
+#pragma unroll
+            for (int c = 0; c < 12; ++c) y[c] = y[c] + xo[c];
+        }
+        // the half spinors of x, as storage holds it, to the neighbouring domains' inboxes
         if (sw + 1 < a.nsweeps) {
-            SV::store(own, y);
+            {
+                cx<C> kept[12];
+#pragma unroll
+                for (int c = 0; c < 12; ++c) kept[c] = y[c];
+                round_spinor<PS, C>(kept);
+                SV::store(own, kept);
+            }
             __syncthreads();
             for (int q = tid; q < ns; q += T) {
                 const int side = q >= ns / 2 ? 1 : 0;
                 const int f = __ldg(a.faces + q - side * (ns / 2)), mu = f >> 10;
                 int t = f & 1023;
-                cx<C> yy[12], k0[3], k1[3];
+                cx<C> xx[12], k0[3], k1[3];
                 long long to;
 #define SAP_SEND(MU, LS_MU, DST)                                                             \
     {                                                                                        \
@@ -573,8 +598,8 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
         } else {                                                                             \
             to = D[MU] > 0 ? dom - DST : dom + (g.nb[MU] - 1) * DST;                         \
         }                                                                                    \
-        SV::load(rsh + SV::at(t), yy);                                                       \
-        face_half<MU, C, LW>(side, yy, lsh, t, k0, k1);                                      \
+        SV::load(rsh + SV::at(t), xx);                                                       \
+        face_half<MU, C, LW>(side, xx, lsh, t, k0, k1);                                      \
     }
                 if (mu == 0)
                     SAP_SEND(0, 1, 1)
@@ -597,21 +622,7 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
                 links_start();
             }
         }
-        // x^l <- x^l + y^l; rho^l is kept for the next visit
-        if (act) {
-            if (!first) {
-                cx<C> xo[12];
-                state_load<C>(xp, g.V, sc, xo);
-#pragma unroll
-                for (int c = 0; c < 12; ++c) y[c] = y[c] + xo[c];
-            }
-            if (last) {
-                store_spinor<PS, C>(xb, g.V, sc, y);
-            } else {
-                store_spinor<CP, C>(xp, g.V, sc, y);
-                store_spinor<CP, C>(rho_g, g.V, sc, rho);
-            }
-        }
+        if (act) store_spinor<PS, C>(xb, g.V, sc, y);
     }
     // the last CTA of this rhs leaves the counters at zero for the next launch
     if (!dead && a.s1 - a.s0 > 1 && tid == 0) {
@@ -691,10 +702,6 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     a.Uimg = w.Uimg;
     a.faces = w.faces;
     a.ns = sap_inbox_slots(g);
-    a.rho = w.rho;
-    a.rho_rs = w.rho_rs;
-    a.xpart = w.xpart;
-    a.xpart_rs = w.xpart_rs;
     a.inbox = w.inbox;
     a.inbox_rs = w.inbox_rs;
     a.jtab = jtab;
@@ -753,19 +760,13 @@ int sap_inbox_slots(const Geom& g) {
 
 int sap_apply_smem(int pspin, int plink, const Geom& g) {
     const int c = (pspin == P64) ? 8 : 4, T = sap_threads(g, 0);
-    const int body = std::max(c * 24 * T, (int)(sap_inbox_bytes(pspin, g) / g.ndom));
-    return body + (int)(sap_link_image_bytes(plink, g, T) / g.ndom) + c * 32 + 16;
+    return c * 24 * T + (int)(sap_link_image_bytes(plink, g, T) / g.ndom) + c * 32 + 16;
 }
 
 // Domains of at most 256 sites whose inbox is no larger than a double-precision
-// field (the scratch that a solve has at hand) and fits in shared memory.
+// field (the scratch that a solve has at hand).
 bool sap_apply_fits(int prec, const Geom& g) {
     return g.B <= 256 && sap_inbox_bytes(prec, g) <= 192 * (size_t)g.V && sap_apply_smem(prec, prec, g) <= 227 * 1024;
-}
-
-size_t sap_state_bytes(int prec, const Geom& g) {
-    const bool half = (prec == P16 || prec == PB16);
-    return (size_t)spinor_bytes(prec == P64 ? P64 : P32, g.V) * (half ? 2 : 1);
 }
 
 size_t sap_inbox_bytes(int prec, const Geom& g) {

@@ -503,10 +503,9 @@ int Solver::step() {
     const FieldRef Lf{vlow, sb, 0, 0};
     const FieldRef Zs = (zp == sp) ? Zf : FieldRef{zsap, sb, 0, 0};  // where the SAP writes z_j
     // z_j = M v_j  (v_j was written in SAP storage to vlow when it was normalised)
-    // The preconditioner's scratch lies in rb (the explicit residual is formed
-    // and consumed within cycle_end, so rb is free during the steps) and in the
-    // staging copy of the right-hand sides: 192 bytes per site and rhs each.
-    if ((rc = sap_run(ctx, sp, U_sap_img, Lf, Zs, rb, fb, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
+    // The preconditioner's scratch lies in the staging copy of the right-hand
+    // sides: 192 bytes per site and rhs.
+    if ((rc = sap_run(ctx, sp, U_sap_img, Lf, Zs, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
         return rc;
     if (zp != sp) {
         ProfScope ps(&ctx->prof, "z_widen", (double)nact * (sb + zb));
