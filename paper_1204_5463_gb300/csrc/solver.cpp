@@ -97,7 +97,7 @@ struct Solver {
     int nblk;
     const char *U_sap_img, *U_mv, *U64;
     // device buffers (owned by the workspace of the context)
-    char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap, *canon;
+    char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap;
     double2 *partial, *dots, *Qd, *etad;
     unsigned *cnt_d, *dcnt_d;  // reduction counters of the multi-axpy and multi-dot launches
     double *norm2d, *scal_d;
@@ -229,9 +229,6 @@ int Solver::setup() {
     if ((rc = W->r.ensure((size_t)nrhs * fb))) return rc;
     if ((rc = W->vlow.ensure((size_t)nrhs * sb))) return rc;
     if (vp != op && (rc = W->rlow.ensure((size_t)nrhs * fv))) return rc;
-    // the caller's layout of the right-hand sides; between the set-up and the
-    // end of a solve it holds the preconditioner's inboxes
-    if ((rc = W->canon.ensure((size_t)nrhs * 24 * V * sizeof(double)))) return rc;
     if ((rc = W->zscr.ensure((size_t)(k > 0 ? k : 1) * zb))) return rc;
     if ((rc = W->partial.ensure((size_t)nrhs * nblk * NP * sizeof(double2)))) return rc;
     // per-rhs counters of the multi-dot and multi-axpy launches (their last CTA
@@ -264,7 +261,6 @@ int Solver::setup() {
     rb = W->r.as<char>();
     vlow = W->vlow.as<char>();
     zscr = W->zscr.as<char>();
-    canon = W->canon.as<char>();
     zsap = (zp != sp) ? W->zsap.as<char>() : nullptr;
     rlow = (vp != op) ? W->rlow.as<char>() : nullptr;
     partial = W->partial.as<double2>();
@@ -503,9 +499,10 @@ int Solver::step() {
     const FieldRef Lf{vlow, sb, 0, 0};
     const FieldRef Zs = (zp == sp) ? Zf : FieldRef{zsap, sb, 0, 0};  // where the SAP writes z_j
     // z_j = M v_j  (v_j was written in SAP storage to vlow when it was normalised)
-    // The preconditioner's scratch lies in the staging copy of the right-hand
-    // sides: 192 bytes per site and rhs.
-    if ((rc = sap_run(ctx, sp, U_sap_img, Lf, Zs, canon, 192 * V, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
+    // The preconditioner's inboxes lie in rb (the explicit residual is formed and
+    // consumed within cycle_end, so rb is free during the steps): fb = 192 bytes
+    // per site and rhs.
+    if ((rc = sap_run(ctx, sp, U_sap_img, Lf, Zs, rb, fb, cols, nrhs, nact, P.sap_cycles, P.mr_steps)))
         return rc;
     if (zp != sp) {
         ProfScope ps(&ctx->prof, "z_widen", (double)nact * (sb + zb));
@@ -627,6 +624,7 @@ int Solver::run(const double* b_user, double* x_user, dw_stats* S, const std::at
     const double* b_dev = b_user;
     double* x_dev = x_user;
     if (P.host_buffers) {
+        if ((rc = W->canon.ensure(canon_bytes))) return rc;
         DW_CUDA_TRY(cudaMemcpyAsync(W->canon.p, b_user, canon_bytes, cudaMemcpyHostToDevice, st));
         b_dev = W->canon.as<double>();
     }
