@@ -37,6 +37,8 @@
 // warps that 128 registers allow, with its pipe busy three quarters of the time;
 // paired, scalar and mixed forms of the hop's FP32 arithmetic are within 2% of one
 // another.
+#include <cuda.h>
+
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -668,6 +670,37 @@ __global__ void faces_kernel(Geom g, unsigned short* faces) {
     }
 }
 
+// SMs that the stream's kernels may use: all, or those of its green context. The
+// driver's functions are asked for by name (the library does not link libcuda);
+// without them, the device's count.
+int stream_sms(cudaStream_t st, int dev, int* sms) {
+    typedef CUresult (*stream_ctx_t)(CUstream, CUcontext*);
+    typedef CUresult (*ctx_resource_t)(CUcontext, CUdevResource*, CUdevResourceType);
+    struct Driver {
+        stream_ctx_t stream_ctx = nullptr;
+        ctx_resource_t ctx_resource = nullptr;
+        Driver() {
+            void *a = nullptr, *b = nullptr;
+            if (cudaGetDriverEntryPointByVersion("cuStreamGetCtx", &a, 12000, cudaEnableDefault) == cudaSuccess &&
+                cudaGetDriverEntryPointByVersion("cuCtxGetDevResource", &b, 12040, cudaEnableDefault) == cudaSuccess) {
+                stream_ctx = reinterpret_cast<stream_ctx_t>(a);
+                ctx_resource = reinterpret_cast<ctx_resource_t>(b);
+            }
+            cudaGetLastError();
+        }
+    };
+    static const Driver d;
+    CUcontext ctx = nullptr;
+    CUdevResource res;
+    if (d.stream_ctx && d.ctx_resource && d.stream_ctx(reinterpret_cast<CUstream>(st), &ctx) == CUDA_SUCCESS &&
+        d.ctx_resource(ctx, &res, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS) {
+        *sms = (int)res.sm.smCount;
+        return DW_OK;
+    }
+    DW_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+    return DW_OK;
+}
+
 template <int PS, int PL, class C>
 int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab, int nrhs,
                 int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof, double bytes_first,
@@ -676,23 +709,23 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     const size_t smem = (size_t)sap_apply_smem(PS, PL, g);
     const void* fn = cl ? (const void*)sap_apply_kernel<PS, PL, C, true> : (const void*)sap_apply_kernel<PS, PL, C, false>;
     // per device and CTA shape: the shared-memory limit is raised once, and the
-    // CTAs that the device holds at a time are asked for once
+    // CTAs that an SM holds at a time are asked for once
     static std::mutex mu;
     static std::map<std::pair<int, std::pair<const void*, std::pair<int, size_t>>>, int> resident;
-    int dev = 0, fit = 0;
+    int dev = 0, fit = 0, sms = 0, rc;
     DW_CUDA_TRY(cudaGetDevice(&dev));
+    if ((rc = stream_sms(st, dev, &sms))) return rc;
     {
         std::lock_guard<std::mutex> lock(mu);
         const auto key = std::make_pair(dev, std::make_pair(fn, std::make_pair(threads, smem)));
         auto it = resident.find(key);
         if (it == resident.end()) {
-            int sms = 0, per = 0;
+            int per = 0;
             DW_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            DW_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             DW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem));
-            it = resident.emplace(key, sms * per).first;
+            it = resident.emplace(key, per).first;
         }
-        fit = it->second;
+        fit = sms * it->second;
     }
     SapArgs<C> a;
     a.g = g;
@@ -723,24 +756,30 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void* args[] = {&a};
+    int sw = 0;
     if ((long long)cfg.gridDim.x <= fit) {
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
         // at most 256 sweeps a launch: the barrier's counter stays small and no
         // launch holds the device for long, however many cycles are asked for
-        for (int sw = 0; sw < a.nsweeps; sw = a.s1) {
+        for (; sw < a.nsweeps; sw = a.s1) {
             a.s0 = sw;
             a.s1 = std::min(a.nsweeps, sw + 256);
             const double bytes = (sw ? 0.0 : 2.0 * (bytes_first - bytes_next)) + (a.s1 - a.s0) * bytes_next;
             ProfScope ps(prof, "sap_sweep", bytes, a.s1 - a.s0);
-            DW_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
+            const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+            // refused for want of room: the remaining sweeps take a launch each
+            if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+                cudaGetLastError();
+                break;
+            }
+            DW_CUDA_TRY(e);
             DW_LAUNCH_CHECK();
         }
-        return DW_OK;
     }
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    for (int sw = 0; sw < a.nsweeps; ++sw) {
+    for (; sw < a.nsweeps; ++sw) {
         a.s0 = sw;
         a.s1 = sw + 1;
         ProfScope ps(prof, "sap_sweep", sw < 2 ? bytes_first : bytes_next);
