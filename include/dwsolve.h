@@ -219,6 +219,11 @@ int dw_residual_history(dw_ctx* ctx, int rhs, double* out, int max, int* n);
  * widened to FP64 (basis format outer_prec, Z in its storage format). */
 int dw_debug_basis(dw_ctx* ctx, int rhs, double* V_out, double* Z_out, double* H_out, int max_cols, int* ncols);
 
+/* Test hook: the limit, in nanoseconds, of a SAP domain's wait for the previous
+ * sweep (negative: the default). A wait that gives up ends the call with
+ * DW_ETIMEOUT; the next one starts afresh. */
+int dw_debug_sap_wait(dw_ctx* ctx, long long ns);
+
 /* Message describing the last error on the calling thread ("" if none). */
 const char* dw_last_error(void);
 

@@ -87,6 +87,7 @@ _SIGS = {
     "dw_last_error": ([], ctypes.c_char_p),
     "dw_cancel": ([_P], _I),
     "dw_debug_basis": ([_P, _I, _P, _P, _P, _I, ctypes.POINTER(_I)], _I),
+    "dw_debug_sap_wait": ([_P, ctypes.c_longlong], _I),
     "dw_residual_history": ([_P, _I, _P, _I, ctypes.POINTER(_I)], _I),
     "dw_profile": ([_P, _I], _I),
     "dw_kernel_launches": ([], ctypes.c_longlong),
@@ -215,6 +216,11 @@ def dw_debug_basis(ctx, rhs: int, V_out=None, Z_out=None, H_out=None, max_cols: 
     _check(_lib.dw_debug_basis(ctx, int(rhs), _ptr(V_out), _ptr(Z_out), _ptr(H_out), int(max_cols), ctypes.byref(n)),
            "dw_debug_basis")
     return n.value
+
+
+def dw_debug_sap_wait(ctx, ns: int) -> None:
+    """Test hook: limit of a SAP domain's wait for the previous sweep (negative: the default)."""
+    _check(_lib.dw_debug_sap_wait(ctx, int(ns)), "dw_debug_sap_wait")
 
 
 def dw_residual_history(ctx, rhs: int = 0):

@@ -193,6 +193,7 @@ int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, cha
         w.inbox = inbox;
         w.inbox_rs = inbox_rs;
         w.err = ctx->sap_err.d;
+        w.wait_ns = ctx->sap_wait_ns;
         if ((rc = sap_tables_for(ctx, &w.faces, &w.bar))) return rc;
         return launch_sap_apply(prec, g, ctx->m0, v, x, w, jtab, nrhs, ncycles, nmr, ctx->stream, ctx->clover(),
                                 &ctx->prof, first, next);
@@ -378,6 +379,12 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     if ((rc = launch_from_internal(storage, ctx->work_out.as<char>(), z, V, nrhs, ctx->stream))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     return sap_check(ctx);
+}
+
+int dw_debug_sap_wait(dw_ctx* ctx, long long ns) {
+    if (!ctx) return fail(DW_EINVAL, "null context");
+    ctx->sap_wait_ns = ns < 0 ? SapWork::kWait : (unsigned long long)ns;
+    return DW_OK;
 }
 
 void dw_default_params(dw_solver_params* P) {

@@ -147,6 +147,7 @@ struct dw_ctx {
     int Uimg_threads[4] = {0, 0, 0, 0};  // CTA size the image was packed for (0: none)
     dwk::HostFlag sap_err;          // set by a SAP kernel whose bounded wait gave up
     dwk::DevBuf sap_faces;          // inbox slots of a domain (launch_sap_faces), with the barrier counters behind them
+    unsigned long long sap_wait_ns = 2000000000ULL;  // SapWork::kWait, unless dw_debug_sap_wait changed it
     bool sap_counters_ok = false;   // the barrier counters are zero (cleared after a wait that gave up)
     dwk::DevBuf work_sap;           // scratch of sap_precondition
     std::atomic<int> cancel{0};     // set by dw_cancel; the running solve stops before its next step
@@ -206,6 +207,8 @@ struct SapWork {
     long long inbox_rs;
     unsigned* bar;
     int* err;
+    unsigned long long wait_ns;  // limit of a wait for the previous sweep
+    static constexpr unsigned long long kWait = 2000000000ULL;
 };
 bool sap_apply_fits(int prec, const Geom& g);
 int sap_apply_smem(int pspin, int plink, const Geom& g);

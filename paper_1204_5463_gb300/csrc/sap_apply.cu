@@ -279,18 +279,12 @@ __device__ __forceinline__ void cta_sum3(C& a, C& b, C& c, C* red) {
 
 // waits until *cnt reaches target, giving up after limit ns
 __device__ __forceinline__ bool count_wait(const unsigned* cnt, unsigned target, unsigned long long limit) {
-    unsigned long long t0 = 0;
+    const unsigned long long t0 = global_ns();
     for (unsigned it = 1;; ++it) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
         if (v >= target) return true;
-        if ((it & 255) == 0) {
-            const unsigned long long now = global_ns();
-            if (t0 == 0)
-                t0 = now;
-            else if (now - t0 > limit)
-                return false;
-        }
+        if ((it & 255) == 0 && global_ns() - t0 > limit) return false;
     }
 }
 
@@ -742,9 +736,10 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     a.nmr = nmr;
     a.nsweeps = 2 * ncycles;
     a.clov = cl ? ((sizeof(C) == 4) ? cl->a32 : cl->a64) : nullptr;
-    // two seconds, and more than an MR step takes in any precision (70 us in FP64)
-    // for each of the steps by which another domain may be behind
-    a.wait_ns = 2000000000ULL + 200000ULL * (unsigned long long)nmr;
+    // two seconds unless the context says otherwise, and more than an MR step takes in
+    // any precision (70 us in FP64) for each of the steps by which another domain may be
+    // behind
+    a.wait_ns = w.wait_ns == SapWork::kWait ? w.wait_ns + 200000ULL * (unsigned long long)nmr : w.wait_ns;
     a.bar = w.bar;
     a.err_host = w.err;
     cudaLaunchConfig_t cfg = {};
