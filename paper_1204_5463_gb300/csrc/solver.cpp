@@ -752,8 +752,13 @@ int solve(dw_ctx* ctx, const double* b, double* x, const dw_solver_params* P, dw
           const std::atomic<int>* cancel) {
     Solver s(ctx, *P);
     int rc = s.setup();
-    if (rc) return rc;
-    return s.run(b, x, S, cancel);
+    if (rc == DW_OK) rc = s.run(b, x, S, cancel);
+    // an error may leave the loop with work in flight; calls return when theirs is done
+    if (rc != DW_OK) {
+        cudaStreamSynchronize(ctx->stream);
+        if (ctx->ws && ctx->ws->back) cudaStreamSynchronize(ctx->ws->back);
+    }
+    return rc;
 }
 
 int residual_history(dw_ctx* ctx, int rhs, double* out, int max, int* n) {
