@@ -259,8 +259,8 @@ __global__ void __launch_bounds__(kThreads, dw_min_blocks<PI, PO, PL, C>())
 // 48: FP32 one field 64 + 32 -> 81 us (HBM and latency), twelve FP16 fields 565
 // + 280 -> 722 us (three CTAs an SM; two 790, and two fields a thread sharing
 // the decoded links 719; instructions: 24 conversions and 24 scalings of every
-// neighbour); FP64 at 16^3 x 32 318 + 10 -> 232 us with hop_pair (the FP64 pipe:
-// 840 instructions a site take 190 us).
+// neighbour); FP64 at 16^3 x 32 318 + 10 -> 250 us with hop_pair (the FP64 pipe:
+// 888 instructions a site take 201 us).
 template <int P, class C, bool CLOV>
 __global__ void __launch_bounds__(kThreads, sizeof(C) == 4 ? 3 : 1)
     dw_out_kernel(Geom g, C diag, const char* in, long long in_rs, double* canon, const char* U, int nrhs,
