@@ -145,14 +145,17 @@ HostFlag::~HostFlag() {
     if (h) cudaFreeHost(h);
 }
 
-int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char** img) {
+int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, char** img) {
     int rc;
     if ((rc = gauge_for(ctx, prec, U))) return rc;
     if ((rc = ctx->sap_err.ensure())) return rc;
     threads = sap_threads(ctx->g, threads);
     if (ctx->Uimg_threads[prec] != threads) {
-        if ((rc = ctx->Uimg[prec].ensure(sap_link_image_bytes(prec, ctx->g, threads)))) return rc;
-        rc = sap_apply_fits(prec, ctx->g)
+        const bool fits = sap_apply_fits(prec, ctx->g);
+        if ((rc = ctx->Uimg[prec].ensure(fits ? sap_apply_image_bytes(prec, ctx->g)
+                                              : sap_link_image_bytes(prec, ctx->g, threads))))
+            return rc;
+        rc = fits
                  ? launch_sap_apply_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), ctx->stream)
                  : launch_sap_link_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), threads, ctx->stream);
         if (rc) return rc;
@@ -162,31 +165,12 @@ int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char
     return DW_OK;
 }
 
-// the table of inbox slots and, behind it, the barrier counters
-static int sap_tables_for(dw_ctx* ctx, const unsigned short** faces, unsigned** bar) {
-    const size_t fbytes = ((size_t)sap_inbox_slots(ctx->g) / 2 * sizeof(unsigned short) + 15) / 16 * 16;
-    const size_t cbytes = 2 * DW_MAX_RHS * sizeof(unsigned);
-    int rc;
-    if (!ctx->sap_faces.p) {
-        if ((rc = ctx->sap_faces.ensure(fbytes + cbytes))) return rc;
-        if ((rc = launch_sap_faces(ctx->g, ctx->sap_faces.as<unsigned short>(), ctx->stream))) return rc;
-    }
-    *faces = ctx->sap_faces.as<unsigned short>();
-    *bar = reinterpret_cast<unsigned*>(ctx->sap_faces.as<char>() + fbytes);
-    if (!ctx->sap_counters_ok) {
-        DW_CUDA_TRY(cudaMemsetAsync(*bar, 0, cbytes, ctx->stream));
-        ctx->sap_counters_ok = true;
-    }
-    return DW_OK;
-}
-
-int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* inbox,
+int sap_run(dw_ctx* ctx, int prec, char* Uimg, FieldRef v, FieldRef x, char* inbox,
             long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr) {
     const Geom& g = ctx->g;
     const long long sb = spinor_bytes(prec, g.V);
     const double first = 0.5 * ((double)nact * 2.0 * sb + link_bytes(prec, g.V));
     const double next = 0.5 * ((double)nact * 3.0 * sb + link_bytes(prec, g.V));
-    int rc;
     if (sap_apply_fits(prec, g)) {
         SapWork w;
         w.Uimg = Uimg;
@@ -194,11 +178,11 @@ int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, cha
         w.inbox_rs = inbox_rs;
         w.err = ctx->sap_err.d;
         w.wait_ns = ctx->sap_wait_ns;
-        if ((rc = sap_tables_for(ctx, &w.faces, &w.bar))) return rc;
         return launch_sap_apply(prec, g, ctx->m0, v, x, w, jtab, nrhs, ncycles, nmr, ctx->stream, ctx->clover(),
                                 &ctx->prof, first, next);
     }
     const int thr = ctx->sap_threads[prec];
+    int rc;
     for (int cyc = 0; cyc < ncycles; ++cyc)
         for (int colour = 0; colour < 2; ++colour) {
             const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
@@ -213,7 +197,7 @@ int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, cha
 int sap_check(dw_ctx* ctx) {
     if (!ctx->sap_err.h || *reinterpret_cast<volatile int*>(ctx->sap_err.h) == 0) return DW_OK;
     *reinterpret_cast<volatile int*>(ctx->sap_err.h) = 0;
-    ctx->sap_counters_ok = false;
+    for (int& t : ctx->Uimg_threads) t = 0;  // the next application's pack sets the counters to zero
     return fail(DW_ETIMEOUT, "a bounded wait of the SAP preconditioner gave up");
 }
 
@@ -264,7 +248,7 @@ int dw_create(const dw_lattice* L, void* cuda_stream, dw_ctx** out) {
         return fail(DW_ECUDA, std::string("no CUDA device: ") + cudaGetErrorString(e));
     }
     c->sap_threads.assign(4, 0);
-    for (auto* b : {&c->U[0], &c->U[1], &c->U[2], &c->U[3], &c->U[4], &c->work_in, &c->work_out, &c->work_aux, &c->work_sap, &c->sap_faces,
+    for (auto* b : {&c->U[0], &c->U[1], &c->U[2], &c->U[3], &c->U[4], &c->work_in, &c->work_out, &c->work_aux,
                    &c->Uimg[0], &c->Uimg[1], &c->Uimg[2], &c->Uimg[3]})
         b->st = c->stream;
     *out = c;
@@ -364,17 +348,19 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     const long long V = ctx->g.V;
     const long long fb = spinor_bytes(storage, V);
     int rc;
-    const char *U, *Uimg;
+    const char* U;
+    char* Uimg;
     // the image is packed before the conversion's launch, not right before the sweeps (sap_run)
     if ((rc = sap_links_for(ctx, storage, ctx->sap_threads[storage], &U, &Uimg))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
-    if ((rc = ctx->work_out.ensure((size_t)nrhs * fb))) return rc;
-    const size_t ibytes = sap_inbox_bytes(storage, ctx->g);
-    if (sap_apply_fits(storage, ctx->g) && (rc = ctx->work_sap.ensure((size_t)nrhs * ibytes))) return rc;
+    // the result and, behind it, the inboxes
+    const size_t zbytes = ((size_t)nrhs * fb + 255) / 256 * 256;
+    const size_t ibytes = sap_apply_fits(storage, ctx->g) ? sap_inbox_bytes(storage, ctx->g) : 0;
+    if ((rc = ctx->work_out.ensure(zbytes + nrhs * ibytes))) return rc;
     if ((rc = launch_to_internal(storage, v, ctx->work_in.as<char>(), V, nrhs, ctx->stream))) return rc;
     FieldRef fv{ctx->work_in.as<char>(), fb, 0, 0}, fx{ctx->work_out.as<char>(), fb, 0, 0};
-    if ((rc = sap_run(ctx, storage, Uimg, fv, fx, ctx->work_sap.as<char>(), (long long)ibytes, nullptr, nrhs, nrhs,
-                      ncycles, nmr)))
+    if ((rc = sap_run(ctx, storage, Uimg, fv, fx, ctx->work_out.as<char>() + zbytes, (long long)ibytes, nullptr, nrhs,
+                      nrhs, ncycles, nmr)))
         return rc;
     if ((rc = launch_from_internal(storage, ctx->work_out.as<char>(), z, V, nrhs, ctx->stream))) return rc;
     DW_CUDA_TRY(cudaStreamSynchronize(ctx->stream));

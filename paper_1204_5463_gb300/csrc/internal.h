@@ -146,10 +146,7 @@ struct dw_ctx {
     dwk::DevBuf Uimg[4];            // SAP links per domain as shared-memory images (per storage precision)
     int Uimg_threads[4] = {0, 0, 0, 0};  // CTA size the image was packed for (0: none)
     dwk::HostFlag sap_err;          // set by a SAP kernel whose bounded wait gave up
-    dwk::DevBuf sap_faces;          // inbox slots of a domain (launch_sap_faces), with the barrier counters behind them
     unsigned long long sap_wait_ns = 2000000000ULL;  // SapWork::kWait, unless dw_debug_sap_wait changed it
-    bool sap_counters_ok = false;   // the barrier counters are zero (cleared after a wait that gave up)
-    dwk::DevBuf work_sap;           // scratch of sap_precondition
     std::atomic<int> cancel{0};     // set by dw_cancel; the running solve stops before its next step
     const dwk::ClovRef* clover() const { return csw != 0.0 ? &clov : nullptr; }
 };
@@ -196,16 +193,14 @@ size_t sap_link_image_bytes(int plink, const Geom& g, int threads);
 int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, int threads, cudaStream_t st);
 // links of precision prec in both layouts for a sweep of `threads` threads
 // (the image is packed on first use and after dw_set_gauge), and the error flag
-int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, const char** img);
+int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, char** img);
 // ----- sap_apply.cu --------------------------------------------------------
 // z = M v with the domains' halos exchanged as half spinors (sap_apply.cu), for
 // domains that sap_apply_fits accepts. inbox: scratch per right-hand side.
 struct SapWork {
-    const char* Uimg;
-    const unsigned short* faces;
+    char* Uimg;  // of launch_sap_apply_image, with the face table and the counters behind the links
     char* inbox;
     long long inbox_rs;
-    unsigned* bar;
     int* err;
     unsigned long long wait_ns;  // limit of a wait for the previous sweep
     static constexpr unsigned long long kWait = 2000000000ULL;
@@ -213,8 +208,12 @@ struct SapWork {
 bool sap_apply_fits(int prec, const Geom& g);
 int sap_apply_smem(int pspin, int plink, const Geom& g);
 int sap_inbox_slots(const Geom& g);
+// the packed links, the table of inbox slots and the barrier counters, at zero (they
+// are left at zero by an application, except by one whose wait gave up)
+size_t sap_apply_image_bytes(int prec, const Geom& g);
+unsigned short* sap_apply_faces(int prec, const Geom& g, char* img);
+unsigned* sap_apply_counters(int prec, const Geom& g, char* img);
 int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st);
-int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st);
 int launch_sap_apply(int prec, const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab,
                      int nrhs, int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof,
                      double bytes_first, double bytes_next);
@@ -228,7 +227,7 @@ size_t sap_inbox_bytes(int prec, const Geom& g);
 // or copy of the stream: the first sweep is launched programmatically and reads the
 // image before it waits for the kernel in front of it, so that kernel must not
 // be the one that writes the image.
-int sap_run(dw_ctx* ctx, int prec, const char* Uimg, FieldRef v, FieldRef x, char* inbox,
+int sap_run(dw_ctx* ctx, int prec, char* Uimg, FieldRef v, FieldRef x, char* inbox,
             long long inbox_rs, RhsCols jtab, int nrhs, int nact, int ncycles, int nmr);
 // after the stream was synchronised: DW_ETIMEOUT if a SAP kernel's bounded wait gave up
 int sap_check(dw_ctx* ctx);

@@ -630,11 +630,24 @@ __global__ void __launch_bounds__(256, sizeof(C) == 4 ? 2 : 1) sap_apply_kernel(
     }
 }
 
-// the links of domain blockIdx.x (both colours) as LinkWarp keeps them in shared memory
+// The links of domain blockIdx.x (both colours) as LinkWarp keeps them in shared
+// memory. Block 0 also writes what follows the image: faces[q], the lower-face site |
+// mu << 10 of inbox slot q (and of its mirror q + ns / 2), and the counters at zero.
 template <int PL>
-__global__ void warp_image_kernel(Geom g, const char* __restrict__ U, char* __restrict__ img) {
+__global__ void warp_image_kernel(Geom g, const char* __restrict__ U, char* __restrict__ img, unsigned short* faces,
+                                  unsigned* bar) {
     const int t = threadIdx.x;
+    if (blockIdx.x == 0 && t < 2 * DW_MAX_RHS) bar[t] = 0u;
     if (t >= g.B) return;
+    if (blockIdx.x == 0) {
+        int ls = 1, off = 0;
+        for (int mu = 0; mu < 4; ++mu) {
+            if ((t / ls) % g.b[mu] == 0)  // the slots run over the other three coordinates in order
+                faces[off + t % ls + ls * (t / (ls * g.b[mu]))] = (unsigned short)(t | (mu << 10));
+            off += g.B / g.b[mu];
+            ls *= g.b[mu];
+        }
+    }
     int D[4], q = blockIdx.x;
     D[0] = q % g.nb[0];
     q /= g.nb[0];
@@ -650,18 +663,6 @@ __global__ void warp_image_kernel(Geom g, const char* __restrict__ U, char* __re
     xg[3] = D[3] * g.b[3] + r;
     LinkWarp<PL>::pack(reinterpret_cast<unsigned char*>(img) + (size_t)blockIdx.x * LinkWarp<PL>::kWarp * (blockDim.x >> 5),
                        t, U, g.V, site_index(g, xg));
-}
-
-// faces[q]: lower-face site | mu << 10 of inbox slot q (and of its mirror q + ns / 2)
-__global__ void faces_kernel(Geom g, unsigned short* faces) {
-    int ls = 1, off = 0;
-    for (int mu = 0; mu < 4; ++mu) {
-        for (int t = threadIdx.x; t < g.B; t += blockDim.x)
-            if ((t / ls) % g.b[mu] == 0)  // the slots run over the other three coordinates in order
-                faces[off + t % ls + ls * (t / (ls * g.b[mu]))] = (unsigned short)(t | (mu << 10));
-        off += g.B / g.b[mu];
-        ls *= g.b[mu];
-    }
 }
 
 // SMs that the stream's kernels may use: all, or those of its green context. The
@@ -727,7 +728,7 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     a.v = v;
     a.x = x;
     a.Uimg = w.Uimg;
-    a.faces = w.faces;
+    a.faces = sap_apply_faces(PL, g, w.Uimg);
     a.ns = sap_inbox_slots(g);
     a.inbox = w.inbox;
     a.inbox_rs = w.inbox_rs;
@@ -740,7 +741,7 @@ int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork&
     // any precision (70 us in FP64) for each of the steps by which another domain may be
     // behind
     a.wait_ns = w.wait_ns == SapWork::kWait ? w.wait_ns + 200000ULL * (unsigned long long)nmr : w.wait_ns;
-    a.bar = w.bar;
+    a.bar = sap_apply_counters(PL, g, w.Uimg);
     a.err_host = w.err;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(g.ndom / 2) * (unsigned)nrhs);
@@ -808,24 +809,34 @@ size_t sap_inbox_bytes(int prec, const Geom& g) {
     return (size_t)g.ndom * (prec == P64 ? Half<double>::bytes(ns) : Half<float>::bytes(ns));
 }
 
-int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st) {
-    const int T = sap_threads(g, 0);
-    if (T != g.B) DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(prec, g, T), st));  // rows of idle threads
-    const unsigned nb = (unsigned)g.ndom;
-    if (prec == P64)
-        warp_image_kernel<P64><<<nb, T, 0, st>>>(g, U, img);
-    else if (prec == P32)
-        warp_image_kernel<P32><<<nb, T, 0, st>>>(g, U, img);
-    else if (prec == P16)
-        warp_image_kernel<P16><<<nb, T, 0, st>>>(g, U, img);
-    else
-        warp_image_kernel<PB16><<<nb, T, 0, st>>>(g, U, img);
-    DW_LAUNCH_CHECK();
-    return DW_OK;
+size_t sap_apply_image_bytes(int prec, const Geom& g) {
+    return sap_link_image_bytes(prec, g, 0) + (sap_inbox_slots(g) / 2 * sizeof(unsigned short) + 15) / 16 * 16 +
+           2 * DW_MAX_RHS * sizeof(unsigned);
 }
 
-int launch_sap_faces(const Geom& g, unsigned short* faces, cudaStream_t st) {
-    faces_kernel<<<1, 256, 0, st>>>(g, faces);
+unsigned short* sap_apply_faces(int prec, const Geom& g, char* img) {
+    return reinterpret_cast<unsigned short*>(img + sap_link_image_bytes(prec, g, 0));
+}
+
+unsigned* sap_apply_counters(int prec, const Geom& g, char* img) {
+    return reinterpret_cast<unsigned*>(img + sap_apply_image_bytes(prec, g)) - 2 * DW_MAX_RHS;
+}
+
+int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st) {
+    const int T = sap_threads(g, 0);
+    static_assert(2 * DW_MAX_RHS <= 32, "a counter per thread of the smallest block");
+    if (T != g.B) DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(prec, g, T), st));  // rows of idle threads
+    const unsigned nb = (unsigned)g.ndom;
+    unsigned short* faces = sap_apply_faces(prec, g, img);
+    unsigned* bar = sap_apply_counters(prec, g, img);
+    if (prec == P64)
+        warp_image_kernel<P64><<<nb, T, 0, st>>>(g, U, img, faces, bar);
+    else if (prec == P32)
+        warp_image_kernel<P32><<<nb, T, 0, st>>>(g, U, img, faces, bar);
+    else if (prec == P16)
+        warp_image_kernel<P16><<<nb, T, 0, st>>>(g, U, img, faces, bar);
+    else
+        warp_image_kernel<PB16><<<nb, T, 0, st>>>(g, U, img, faces, bar);
     DW_LAUNCH_CHECK();
     return DW_OK;
 }

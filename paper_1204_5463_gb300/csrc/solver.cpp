@@ -95,7 +95,8 @@ struct Solver {
     long long fv;       // bytes of one basis vector in format vp
     int NP;             // multi-dot row length (m + 2)
     int nblk;
-    const char *U_sap_img, *U_mv, *U64;
+    const char *U_mv, *U64;
+    char* U_sap_img;
     // device buffers (owned by the workspace of the context)
     char *Vb, *Zb, *xb, *bb, *rb, *vlow, *zscr, *rlow, *zsap;
     double2 *partial, *dots, *Qd, *etad;
