@@ -145,21 +145,19 @@ HostFlag::~HostFlag() {
     if (h) cudaFreeHost(h);
 }
 
-int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, char** img) {
+int sap_links_for(dw_ctx* ctx, int prec, const char** U, char** img) {
     int rc;
     if ((rc = gauge_for(ctx, prec, U))) return rc;
     if ((rc = ctx->sap_err.ensure())) return rc;
-    threads = sap_threads(ctx->g, threads);
-    if (ctx->Uimg_threads[prec] != threads) {
+    if (!ctx->Uimg_ready[prec]) {
         const bool fits = sap_apply_fits(prec, ctx->g);
         if ((rc = ctx->Uimg[prec].ensure(fits ? sap_apply_image_bytes(prec, ctx->g)
-                                              : sap_link_image_bytes(prec, ctx->g, threads))))
+                                              : sap_link_image_bytes(prec, ctx->g))))
             return rc;
-        rc = fits
-                 ? launch_sap_apply_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), ctx->stream)
-                 : launch_sap_link_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), threads, ctx->stream);
+        rc = fits ? launch_sap_apply_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), ctx->stream)
+                  : launch_sap_link_image(prec, ctx->g, *U, ctx->Uimg[prec].as<char>(), ctx->stream);
         if (rc) return rc;
-        ctx->Uimg_threads[prec] = threads;
+        ctx->Uimg_ready[prec] = true;
     }
     *img = ctx->Uimg[prec].as<char>();
     return DW_OK;
@@ -181,13 +179,12 @@ int sap_run(dw_ctx* ctx, int prec, char* Uimg, FieldRef v, FieldRef x, char* inb
         return launch_sap_apply(prec, g, ctx->m0, v, x, w, jtab, nrhs, ncycles, nmr, ctx->stream, ctx->clover(),
                                 &ctx->prof, first, next);
     }
-    const int thr = ctx->sap_threads[prec];
     int rc;
     for (int cyc = 0; cyc < ncycles; ++cyc)
         for (int colour = 0; colour < 2; ++colour) {
             const int mode = (cyc > 0) ? 2 : (colour == 0 ? 0 : 1);
             ProfScope ps(&ctx->prof, "sap_sweep", mode == 2 ? next : first);
-            if ((rc = launch_sap_sweep(prec, prec, g, ctx->m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, thr,
+            if ((rc = launch_sap_sweep(prec, prec, g, ctx->m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode,
                                        ctx->stream, ctx->clover(), ctx->sap_err.d)))
                 return rc;
         }
@@ -197,7 +194,7 @@ int sap_run(dw_ctx* ctx, int prec, char* Uimg, FieldRef v, FieldRef x, char* inb
 int sap_check(dw_ctx* ctx) {
     if (!ctx->sap_err.h || *reinterpret_cast<volatile int*>(ctx->sap_err.h) == 0) return DW_OK;
     *reinterpret_cast<volatile int*>(ctx->sap_err.h) = 0;
-    for (int& t : ctx->Uimg_threads) t = 0;  // the next application's pack sets the counters to zero
+    for (bool& ready : ctx->Uimg_ready) ready = false;  // the next application's pack sets the counters to zero
     return fail(DW_ETIMEOUT, "a bounded wait of the SAP preconditioner gave up");
 }
 
@@ -247,7 +244,6 @@ int dw_create(const dw_lattice* L, void* cuda_stream, dw_ctx** out) {
         cudaGetLastError();
         return fail(DW_ECUDA, std::string("no CUDA device: ") + cudaGetErrorString(e));
     }
-    c->sap_threads.assign(4, 0);
     for (auto* b : {&c->U[0], &c->U[1], &c->U[2], &c->U[3], &c->U[4], &c->work_in, &c->work_out, &c->work_aux,
                    &c->Uimg[0], &c->Uimg[1], &c->Uimg[2], &c->Uimg[3]})
         b->st = c->stream;
@@ -283,7 +279,7 @@ int dw_set_gauge(dw_ctx* ctx, const double* U, int on_device) {
     }
     if ((rc = launch_gauge_convert(P64, src, ctx->U[P64].as<char>(), ctx->g.V, ctx->stream))) return rc;
     for (int p = 0; p < 5; ++p) ctx->U_ready[p] = false;
-    for (int p = 0; p < 4; ++p) ctx->Uimg_threads[p] = 0;
+    for (bool& ready : ctx->Uimg_ready) ready = false;
     ctx->U_ready[P64] = true;
     ctx->have_gauge = true;
     if (ctx->csw != 0.0 && (rc = dw_set_clover(ctx, ctx->csw))) return rc;  // the clover term follows the links
@@ -351,7 +347,7 @@ int sap_precondition(dw_ctx* ctx, const double* v, double* z, int ncycles, int n
     const char* U;
     char* Uimg;
     // the image is packed before the conversion's launch, not right before the sweeps (sap_run)
-    if ((rc = sap_links_for(ctx, storage, ctx->sap_threads[storage], &U, &Uimg))) return rc;
+    if ((rc = sap_links_for(ctx, storage, &U, &Uimg))) return rc;
     if ((rc = ctx->work_in.ensure((size_t)nrhs * fb))) return rc;
     // the result and, behind it, the inboxes
     const size_t zbytes = ((size_t)nrhs * fb + 255) / 256 * 256;

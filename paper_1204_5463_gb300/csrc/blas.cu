@@ -353,10 +353,7 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
     if (grp == 0) {
         const double sum = cta_sum(E::nfin(wacc), sh);
         if (t == 0) out[nvmax] = make_double2(sum, 0.0);
-        if (!cnt)
-            for (int i = nv + t; i < nvmax; i += kT) out[i] = make_double2(0.0, 0.0);  // the groups cover [0, nv)
     }
-    if (!cnt) return;
     // the last CTA of each group reduces the group's rows: the groups' sums run
     // side by side, and nobody adds rows that this launch has not got
     if (!last_cta(cnt + r * kMaxGroups + grp, (unsigned)nslots)) return;
@@ -370,27 +367,6 @@ __global__ void __launch_bounds__(kT, 2) multidot_kernel(VecRef Vb, VecRef w, lo
         s = cta_sum(s, sh);
         if (t == 0) fr[nvmax] = make_double2(s, 0.0);
         for (int i = nv + t; i < nvmax; i += kT) fr[i] = make_double2(0.0, 0.0);
-    }
-}
-
-// out[r][i] = sum_blk partial[r][blk][i]: warp i sums its row lane-strided,
-// then a fixed shuffle tree (deterministic)
-__global__ void __launch_bounds__(1024) finalize_kernel(const double2* partial, int nblk, int NP, const __grid_constant__ RhsCols jtab,
-                                                        double2* out) {
-    const int r = blockIdx.x;
-    if (jtab && jtab[r] < 0) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = warp; i < NP; i += 32) {
-        double2 s = make_double2(0.0, 0.0);
-        const double2* p = partial + (long long)r * nblk * NP + i;
-        for (int b = lane; b < nblk; b += 32) {
-            const double2 t = p[(long long)b * NP];
-            s.x += t.x;
-            s.y += t.y;
-        }
-        s.x = warp_sum(s.x);
-        s.y = warp_sum(s.y);
-        if (lane == 0) out[(long long)r * NP + i] = s;
     }
 }
 
@@ -871,10 +847,6 @@ int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, RhsCols jtab, int 
         multidot_kernel<P64><<<grid, kT, multidot_smem<P64>(), st>>>(Vb, w, n, jtab, nv_off, nvmax, ngroups, partial,
                                                                     cnt, out, cols);
     DW_LAUNCH_CHECK();
-    if (!cnt) {  // without counters, a separate reduction launch
-        finalize_kernel<<<nrhs, 1024, 0, st>>>(partial, (int)nb, nvmax + 1, jtab, out);
-        DW_LAUNCH_CHECK();
-    }
     return DW_OK;
 }
 

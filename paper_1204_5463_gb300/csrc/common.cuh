@@ -11,6 +11,8 @@
 
 #include <type_traits>
 
+#include "dwsolve.h"
+
 namespace dwk {
 
 // ---------------------------------------------------------------------------
@@ -760,8 +762,8 @@ __device__ __forceinline__ void clover_acc(const char* A, long long V, long long
 // The column table goes to the kernels by value (their parameters lie in
 // constant memory): a step's launches then wait for no copy.
 struct RhsCols {
-    int on;     // 0: no table, column 0 for every rhs, all active
-    int j[16];  // DW_MAX_RHS
+    int on;  // 0: no table, column 0 for every rhs, all active
+    int j[DW_MAX_RHS];
     __host__ __device__ RhsCols(decltype(nullptr) = nullptr) : on(0) {}
     __host__ __device__ explicit operator bool() const { return on != 0; }
     __host__ __device__ int operator[](int r) const { return j[r]; }

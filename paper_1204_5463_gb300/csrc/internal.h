@@ -138,13 +138,12 @@ struct dw_ctx {
     bool U_ready[5] = {false, false, false, false, false};
     dwk::DevBuf work_in, work_out, work_aux;  // conversions in dw_apply / sap_precondition
     dwk::Profiler prof;
-    std::vector<int> sap_threads;  // tuned launch shape per precision (0 = default)
     dwk::Workspace* ws = nullptr;  // solver workspace, kept between solves
     double csw = 0.0;               // clover coefficient (0: plain Wilson operator)
     dwk::DevBuf clov64, clov32;     // clover term, FP64 [72][V] and FP32 float4 [18][V]
     dwk::ClovRef clov{nullptr, nullptr};
     dwk::DevBuf Uimg[4];            // SAP links per domain as shared-memory images (per storage precision)
-    int Uimg_threads[4] = {0, 0, 0, 0};  // CTA size the image was packed for (0: none)
+    bool Uimg_ready[4] = {false, false, false, false};
     dwk::HostFlag sap_err;          // set by a SAP kernel whose bounded wait gave up
     unsigned long long sap_wait_ns = 2000000000ULL;  // SapWork::kWait, unless dw_debug_sap_wait changed it
     std::atomic<int> cancel{0};     // set by dw_cancel; the running solve stops before its next step
@@ -180,20 +179,19 @@ int launch_clover_compute(const Geom& g, const char* U64, double csw, double* A6
 // One colour half-sweep of SAP (Algorithm 2) on every domain of `colour`:
 // r = v - D x (full operator), nmr MR steps on D^l y = r, x += y.
 // mode 0: x == 0 everywhere (r = v, x = y); 1: x == 0 on this colour; 2: general.
-// Uimg: the links of every domain packed by launch_sap_link_image for the same
-// thread count (the sweep reads its links only there); err_host: HostFlag::d,
-// set if a link copy did not complete.
+// Uimg: the links of every domain packed by launch_sap_link_image (the sweep reads
+// its links only there); err_host: HostFlag::d, set if a link copy did not complete.
 int launch_sap_sweep(int pspin, int plink, const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg,
-                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
+                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, cudaStream_t st,
                      const ClovRef* cl, int* err_host);
-int sap_smem_bytes(int pspin, int plink, const Geom& g, int threads);
-// CTA size of the SAP sweep (threads, or the domain volume rounded up to a warp multiple when 0)
-int sap_threads(const Geom& g, int threads);
-size_t sap_link_image_bytes(int plink, const Geom& g, int threads);
-int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, int threads, cudaStream_t st);
-// links of precision prec in both layouts for a sweep of `threads` threads
-// (the image is packed on first use and after dw_set_gauge), and the error flag
-int sap_links_for(dw_ctx* ctx, int prec, int threads, const char** U, char** img);
+int sap_smem_bytes(int pspin, int plink, const Geom& g);
+// CTA size of the SAP kernels: the domain volume rounded up to a warp multiple
+int sap_threads(const Geom& g);
+size_t sap_link_image_bytes(int plink, const Geom& g);
+int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, cudaStream_t st);
+// links of precision prec in both layouts (the image is packed on first use, after
+// dw_set_gauge and after a wait that gave up), and the error flag
+int sap_links_for(dw_ctx* ctx, int prec, const char** U, char** img);
 // ----- sap_apply.cu --------------------------------------------------------
 // z = M v with the domains' halos exchanged as half spinors (sap_apply.cu), for
 // domains that sap_apply_fits accepts. inbox: scratch per right-hand side.
@@ -246,16 +244,15 @@ struct VecRef {
 // nv_active: the largest number of basis vectors any rhs has in this launch
 // (sizes the grid); nvmax: the row length of partial/out minus one
 // cnt: zeroed counters (left zeroed), kDotCounters per rhs: the last CTA of each
-// group of vectors sums the group's partial rows itself; nullptr: a separate
-// reduction launch. cols (device, one int per rhs, may be null) receives the
+// group of vectors sums the group's partial rows itself. cols (device, one int per rhs, may be null) receives the
 // column table for the multi-axpy after it: reading the table from memory, that
 // kernel's loop is 643 us where every form with the table in its parameters is
 // 664 to 863 us (12 rhs, 16 vectors on average, 16^3 x 32)
 constexpr int kDotCounters = 8;
 int launch_multidot(int vp, VecRef Vb, VecRef w, long long n, RhsCols jtab, int nv_off, int nvmax, int nv_active,
-                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt = nullptr, int* cols = nullptr);
+                    int nrhs, double2* partial, int nblk, double2* out, cudaStream_t st, unsigned* cnt, int* cols = nullptr);
 // w -= sum_i coef[r][i] V_i (i < nv[r]);  out_norm2[r] = ||w||^2 after the update;
-// cnt as above, one counter per rhs; jtab: the device table of the multi-dot
+// cnt: one zeroed counter per rhs (left zeroed); nullptr: a separate reduction launch; jtab: the device table of the multi-dot
 int launch_multiaxpy(int vp, VecRef Vb, VecRef w, long long n, const int* jtab, int nv_off, int nrhs,
                      const double2* coef, int coef_ld, double2* partial, int nblk, double* out_norm2,
                      cudaStream_t st, unsigned* cnt = nullptr);

@@ -454,9 +454,10 @@ __global__ void link_image_kernel(Geom g, const char* __restrict__ U, char* __re
 
 template <int PS, int PL, class C>
 int sap_launch_t(const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg, RhsCols jtab, int nrhs,
-                 int colour, int nmr, int mode, int threads, cudaStream_t st, const ClovRef* cl, int* err_host) {
+                 int colour, int nmr, int mode, cudaStream_t st, const ClovRef* cl, int* err_host) {
+    const int threads = sap_threads(g);
     if (cl && threads > 256) return fail(DW_EINVAL, "the clover SAP sweep handles domains of at most 256 sites");
-    const size_t smem = (size_t)sap_smem_bytes(PS, PL, g, threads);
+    const size_t smem = (size_t)sap_smem_bytes(PS, PL, g);
     // the shared-memory limit is a per-device property of the kernel: set it once per device
     static std::mutex mu;
     static std::set<int> done;
@@ -508,22 +509,21 @@ size_t link_sh_bytes(int plink) { return plink == P64 ? 576 : plink == P32 ? 288
 
 }  // namespace
 
-int sap_smem_bytes(int pspin, int plink, const Geom& g, int threads) {
-    const size_t c = (pspin == P64) ? 8 : 4;
-    (void)g;
+int sap_smem_bytes(int pspin, int plink, const Geom& g) {
+    const size_t c = (pspin == P64) ? 8 : 4, threads = sap_threads(g);
     // rho/x, links, the [32][3] reduction buffer, the links' mbarrier
     return (int)(c * 24 * threads + link_sh_bytes(plink) * threads + c * 3 * 32 + 16);
 }
 
-int sap_threads(const Geom& g, int threads) { return threads > 0 ? threads : ((g.B + 31) / 32) * 32; }
+int sap_threads(const Geom& g) { return ((g.B + 31) / 32) * 32; }
 
-size_t sap_link_image_bytes(int plink, const Geom& g, int threads) {
-    return link_sh_bytes(plink) * (size_t)sap_threads(g, threads) * (size_t)g.ndom;
+size_t sap_link_image_bytes(int plink, const Geom& g) {
+    return link_sh_bytes(plink) * (size_t)sap_threads(g) * (size_t)g.ndom;
 }
 
-int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, int threads, cudaStream_t st) {
-    threads = sap_threads(g, threads);
-    DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(plink, g, threads), st));  // rows of idle threads
+int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, cudaStream_t st) {
+    const int threads = sap_threads(g);
+    DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(plink, g), st));  // rows of idle threads
     const unsigned nb = (unsigned)g.ndom;
     if (plink == P64)
         link_image_kernel<P64><<<nb, threads, 0, st>>>(g, U, img);
@@ -540,24 +540,22 @@ int launch_sap_link_image(int plink, const Geom& g, const char* U, char* img, in
 }
 
 int launch_sap_sweep(int pspin, int plink, const Geom& g, double m0, FieldRef v, FieldRef x, const char* Uimg,
-                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, int threads, cudaStream_t st,
+                     RhsCols jtab, int nrhs, int colour, int nmr, int mode, cudaStream_t st,
                      const ClovRef* cl, int* err_host) {
-    threads = sap_threads(g, threads);
-    if (threads < g.B || threads % 32 != 0 || threads > 1024) return fail(DW_EINVAL, "bad SAP thread count");
-    if (sap_smem_bytes(pspin, plink, g, threads) > 227 * 1024)
+    if (sap_smem_bytes(pspin, plink, g) > 227 * 1024)
         return fail(DW_EINVAL, "SAP domain does not fit in shared memory at this precision");
     if (nmr < 1) return fail(DW_EINVAL, "nmr must be >= 1");
     if (pspin == P64 && plink == P64)
-        return sap_launch_t<P64, P64, double>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, threads, st,
+        return sap_launch_t<P64, P64, double>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, st,
                                               cl, err_host);
     if (pspin == P32 && plink == P32)
-        return sap_launch_t<P32, P32, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, threads, st,
+        return sap_launch_t<P32, P32, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, st,
                                              cl, err_host);
     if (pspin == P16 && plink == P16)
-        return sap_launch_t<P16, P16, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, threads, st,
+        return sap_launch_t<P16, P16, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, st,
                                              cl, err_host);
     if (pspin == PB16 && plink == PB16)
-        return sap_launch_t<PB16, PB16, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, threads, st,
+        return sap_launch_t<PB16, PB16, float>(g, m0, v, x, Uimg, jtab, nrhs, colour, nmr, mode, st,
                                                cl, err_host);
     return fail(DW_EINVAL, "unsupported SAP precision combination");
 }

@@ -700,7 +700,7 @@ template <int PS, int PL, class C>
 int sap_apply_t(const Geom& g, double m0, FieldRef v, FieldRef x, const SapWork& w, RhsCols jtab, int nrhs,
                 int ncycles, int nmr, cudaStream_t st, const ClovRef* cl, Profiler* prof, double bytes_first,
                 double bytes_next) {
-    const int threads = sap_threads(g, 0);
+    const int threads = sap_threads(g);
     const size_t smem = (size_t)sap_apply_smem(PS, PL, g);
     const void* fn = cl ? (const void*)sap_apply_kernel<PS, PL, C, true> : (const void*)sap_apply_kernel<PS, PL, C, false>;
     // per device and CTA shape: the shared-memory limit is raised once, and the
@@ -794,8 +794,8 @@ int sap_inbox_slots(const Geom& g) {
 }
 
 int sap_apply_smem(int pspin, int plink, const Geom& g) {
-    const int c = (pspin == P64) ? 8 : 4, T = sap_threads(g, 0);
-    return c * 24 * T + (int)(sap_link_image_bytes(plink, g, T) / g.ndom) + c * 32 + 16;
+    const int c = (pspin == P64) ? 8 : 4, T = sap_threads(g);
+    return c * 24 * T + (int)(sap_link_image_bytes(plink, g) / g.ndom) + c * 32 + 16;
 }
 
 // Domains of at most 256 sites whose inbox is no larger than a double-precision
@@ -810,12 +810,12 @@ size_t sap_inbox_bytes(int prec, const Geom& g) {
 }
 
 size_t sap_apply_image_bytes(int prec, const Geom& g) {
-    return sap_link_image_bytes(prec, g, 0) + (sap_inbox_slots(g) / 2 * sizeof(unsigned short) + 15) / 16 * 16 +
+    return sap_link_image_bytes(prec, g) + (sap_inbox_slots(g) / 2 * sizeof(unsigned short) + 15) / 16 * 16 +
            2 * DW_MAX_RHS * sizeof(unsigned);
 }
 
 unsigned short* sap_apply_faces(int prec, const Geom& g, char* img) {
-    return reinterpret_cast<unsigned short*>(img + sap_link_image_bytes(prec, g, 0));
+    return reinterpret_cast<unsigned short*>(img + sap_link_image_bytes(prec, g));
 }
 
 unsigned* sap_apply_counters(int prec, const Geom& g, char* img) {
@@ -823,9 +823,9 @@ unsigned* sap_apply_counters(int prec, const Geom& g, char* img) {
 }
 
 int launch_sap_apply_image(int prec, const Geom& g, const char* U, char* img, cudaStream_t st) {
-    const int T = sap_threads(g, 0);
+    const int T = sap_threads(g);
     static_assert(2 * DW_MAX_RHS <= 32, "a counter per thread of the smallest block");
-    if (T != g.B) DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(prec, g, T), st));  // rows of idle threads
+    if (T != g.B) DW_CUDA_TRY(cudaMemsetAsync(img, 0, sap_link_image_bytes(prec, g), st));  // rows of idle threads
     const unsigned nb = (unsigned)g.ndom;
     unsigned short* faces = sap_apply_faces(prec, g, img);
     unsigned* bar = sap_apply_counters(prec, g, img);

@@ -216,7 +216,7 @@ int Solver::setup() {
     nblk = blas_nblk(n);
     int rc;
     const char* U_sap;
-    if ((rc = sap_links_for(ctx, sp, ctx->sap_threads[sp], &U_sap, &U_sap_img))) return rc;
+    if ((rc = sap_links_for(ctx, sp, &U_sap, &U_sap_img))) return rc;
     if ((rc = gauge_for(ctx, mp == P64 ? P64 : P32, &U_mv))) return rc;
     // explicit residual: FP64 links for FP64 outer vectors, double-float links otherwise
     if ((rc = gauge_for(ctx, op == PDF ? PDF : P64, &U64))) return rc;

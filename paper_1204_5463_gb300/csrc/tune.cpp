@@ -48,8 +48,7 @@ std::vector<std::vector<int>> candidates(const int* dims, int sap_prec) {
                     if (vol < 32 || vol > 1024 || mx > 2 * mn) continue;
                     dwk::Geom g{};
                     g.B = vol;
-                    const int threads = ((vol + 31) / 32) * 32;
-                    if (dwk::sap_smem_bytes(sap_prec, sap_prec, g, threads) > 227 * 1024) continue;
+                    if (dwk::sap_smem_bytes(sap_prec, sap_prec, g) > 227 * 1024) continue;
                     out.push_back({a, b, c, d});
                 }
     // time only the twelve candidates closest to 256-site domains (the
