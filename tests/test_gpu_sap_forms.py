@@ -2,7 +2,8 @@
 result against the oracle: the application split over two cooperative launches
 (260 sweeps) in FP32 and FP64, FP64 over several cycles with several right-hand
 sides and the clover term, one launch per sweep when the domains exceed what the
-device holds at a time, and the domains that run the stand-alone sweep.
+device holds at a time, the domains that run the stand-alone sweep, and domains one
+site thick in the application kernel.
 
 A call launches one conversion in, the application and one conversion out.
 Tolerances in the 2-norm as in the parity tests (FP64 1e-11, FP32 4 u). The 260
@@ -26,6 +27,11 @@ CASES = [
     ((8, 8, 8, 8), (4, 4, 4, 4), 4, 3, 3, 1.0, "f32", 1),
     ((16, 16, 16, 16), (4, 4, 4, 4), 3, 2, 2, 0.0, "f64", 6),    # 256 CTAs of one an SM
     ((8, 8, 8, 8), (4, 4, 4, 2), 3, 2, 1, 1.0, "f64", 6),        # the stand-alone sweep
+    # one site in a direction: both its faces there are the same site
+    ((4, 8, 8, 8), (1, 4, 4, 4), 3, 2, 2, 0.0, "f32", 1),
+    ((8, 4, 8, 8), (4, 1, 4, 4), 3, 2, 1, 1.0, "f32", 1),
+    ((8, 8, 4, 8), (4, 4, 1, 4), 3, 2, 1, 0.0, "f32", 1),
+    ((8, 8, 8, 2), (4, 4, 4, 1), 3, 2, 1, 1.0, "f32", 1),
 ]
 
 
